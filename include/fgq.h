@@ -251,9 +251,11 @@ fgq_status fgq_quantize_weights_w8(const float* w, int M, int Kred, int8_t* wq, 
  * The fp32 result is within 1e-5 * act_scale * sum_g |alpha_g * s_g| of the exact value.
  * Memory: the tensor-core kernels take per-call temporaries from a library-owned
  * stream-ordered pool of the current device and return them on the same stream: the
- * activations as fp16 (2 bytes per element read), and the ternary operand -- at G >= 64
- * the codes as fp16 (2 * M * Kp bytes), at G = 4 its block-diagonal form (4 * 2 * M' * Kp
- * bytes per fp16 part, two parts for fp32 alphas, M' = M rounded up to 32 per conv group).
+ * activations as fp16 (2 bytes per element read; for G < 64 each conv group's channels padded
+ * to a multiple of 64), and the ternary operand -- at G >= 64 the codes as fp16 (2 * M * Kp
+ * bytes), for G < 64 the folded weights (two fp16 parts, and room for the parts that widely
+ * spread alphas need: 8 * M' * Kp' bytes, M' and Kp' padded to multiples of 64; the group sums
+ * of G = 4 take 8 * M' * Kp bytes for a block-diagonal form instead).
  * The pool keeps freed blocks, so only a call that needs more than the pool holds reaches
  * the device allocator.  The dp4a and few-row paths allocate nothing.
  * Errors: FGQ_ERR_ARG (null pointers, bad sizes, Kred odd for 4-bit types),

@@ -20,12 +20,15 @@ extern "C" {
 typedef enum {
   FGQ_PATH_AUTO = 0,   /* choose per shape: the few-row path for small GEMMs; with
                           fixed-point alphas the dense tensor-core path where it applies;
-                          else the tensor cores where the shape is covered (G = 4 only with
-                          at least 64 filters per conv group), else the CUDA cores */
+                          else the tensor cores where the shape is covered (G < 64 only with
+                          at least 64 filters and 16 channels per conv group, and not the
+                          smallest layers), else the CUDA cores */
   FGQ_PATH_SIMT = 1,   /* CUDA-core path: dp4a group sums, one FMA per group */
   FGQ_PATH_TC = 2,     /* tensor-core path (tcgen05): G in {64, 128} with K-tiles aligned to
-                          the group; G = 4 with a block-diagonal activation operand
-                          (Cg a multiple of 64) */
+                          the group; smaller G with the alphas folded into integer weights on a
+                          common grid per 256 reduction elements (two fp16 parts).  Forced: G in
+                          {4, 64, 128} with Cg a multiple of 64; the automatic choice also takes
+                          it for G = 8, 16, 32 and other channel counts */
   FGQ_PATH_GEMV = 3,   /* few-row path for GEMMs with P <= 8 (8-bit activations, Kred a
                           multiple of 16, G >= 4): one warp per filter row streams the
                           weights once; the automatic choice for such calls */
@@ -71,10 +74,9 @@ int64_t fgq_debug_set_wait_limit_us(int64_t us);
 int fgq_debug_allow_split_fold(int allow);
 
 /*
- * Runs the G = 4 tensor-core output kernel of this thread's calls on CTA pairs (on != 0: two
- * SMs share each 64-filter x 256-position tile through cta_group::2 MMAs) or on single CTAs
- * (0, the default: 32-filter tiles), the same results either way.  Returns the previous
- * setting.
+ * Remembered per thread and returned by the next call; no kernel depends on it (the CTA-pair
+ * form of the G = 4 kernel that it used to select is gone: every contraction kernel runs on
+ * single CTAs).  Returns the previous setting.
  */
 int fgq_debug_cta_pairs(int on);
 

@@ -25,7 +25,7 @@ thread_local int t_last_path = FGQ_PATH_AUTO;
 thread_local int64_t t_wait_limit_us = -1;
 thread_local int t_split_fold = 0;
 thread_local int t_last_cuda_error = 0;  // cudaError_t of the last failed launch on this thread
-thread_local int t_cta_pairs = 0;        // G = 4 output kernel on CTA pairs (off: single CTAs)
+thread_local int t_cta_pairs = 0;        // remembered only: every contraction kernel runs on single CTAs
 thread_local int t_max_ksplit = 8;       // group ranges a G >= 64 tile may be split into
 thread_local int t_last_ksplit = 0;      // ranges of this thread's last G >= 64 tensor-core call
 
@@ -71,10 +71,25 @@ bool tc_any(const Geom& g) { return g.G == 4 ? tc4_supports(g) : tc_supports(g);
 
 bool gemv_any(const Geom& g) { return !g.is_conv && gemv_supports((int)g.P, g.Kred, g.G, g.act_type); }
 
-// Fewest filters per conv group for which the automatic choice sends a G = 4 layer to the
-// tensor cores (a 64-filter layer fills half of the 128-row tile and still runs at about
-// twice the dp4a kernel's rate).
-constexpr int T4_MIN_FILTERS = 64;
+// Layers with G < 64 that the automatic choice leaves to the dp4a kernel: fewer filters or
+// channels per conv group than fill a 64 x 64 weight image by a fair part, and layers so small
+// that dp4a, which needs no operand preparation, is done first -- its time is about 0.05 us per
+// reduction element and wave of 64 x 128 output blocks (two blocks per SM), against two launches:
+// one wave of Kred = 256 17 us a call against 23 us, of Kred = 432 33 us against 25 us, of
+// Kred = 1024 54 us against 22 us (calls back to back, host work included).
+constexpr int FOLD_MIN_FILTERS = 64;
+constexpr int FOLD_MIN_CHANNELS = 16;
+constexpr int64_t SIMT_WAVE_KRED = 256;
+constexpr int TC_MIN_G = 64;  // from here on a group fills an MMA K-tile
+
+bool fold_any(const Geom& g) {
+  if (g.Mg < FOLD_MIN_FILTERS || g.Cg < FOLD_MIN_CHANNELS || !fold_supports(g)) return false;
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t blocks = (g.P + 127) / 128 * ((g.Mg + 63) / 64) * g.groups;
+  return (blocks + 2 * sms - 1) / (2 * sms) * g.Kred > SIMT_WAVE_KRED;
+}
 
 int choose_path(const Geom& g, bool sums, bool qa) {
   const int forced = t_path;
@@ -84,7 +99,7 @@ int choose_path(const Geom& g, bool sums, bool qa) {
     if (forced == FGQ_PATH_GEMV || forced == FGQ_PATH_DENSE) return -1;
     if (forced == FGQ_PATH_SIMT) return FGQ_PATH_SIMT;
     if (forced == FGQ_PATH_TC) return tc_any(g) ? FGQ_PATH_TC : -1;
-    if (g.G == 4 && g.Mg < T4_MIN_FILTERS) return FGQ_PATH_SIMT;
+    if (g.G == 4 && g.Mg < FOLD_MIN_FILTERS) return FGQ_PATH_SIMT;
     return tc_any(g) ? FGQ_PATH_TC : FGQ_PATH_SIMT;
   }
   if (forced == FGQ_PATH_SIMT) return FGQ_PATH_SIMT;
@@ -96,11 +111,8 @@ int choose_path(const Geom& g, bool sums, bool qa) {
   if (gemv_any(g)) return FGQ_PATH_GEMV;  // a few activation rows: stream the weights once
   // fixed-point alphas fold exactly into fp16 weights: one dense tensor-core contraction
   if (qa && dense_supports(g)) return FGQ_PATH_DENSE;
-  // automatic choice: the tensor cores where the shape is covered, except G = 4 layers with
-  // fewer than T4_MIN_FILTERS filters per conv group, where most rows of the 128-row MMA
-  // tile would sit idle and the dp4a kernel is faster
-  if (g.G == 4 && g.Mg < T4_MIN_FILTERS) return FGQ_PATH_SIMT;
-  return tc_any(g) ? FGQ_PATH_TC : FGQ_PATH_SIMT;
+  // automatic choice: the tensor cores where the shape is covered
+  return (g.G < TC_MIN_G ? fold_any(g) : tc_any(g)) ? FGQ_PATH_TC : FGQ_PATH_SIMT;
 }
 
 // Fixed-point alphas of a contraction call (nullptr: fp32 alphas).
@@ -139,8 +151,9 @@ fgq_status contract(const void* act, const Geom& g, const uint32_t* codes, const
   }
   fgq_status st;
   if (path == FGQ_PATH_TC)
-    st = g.G == 4 ? launch_tc4_contract(act, g, codes, alpha, act_scale, out, sums, err, s)
-                  : launch_tc_contract(act, g, codes, alpha, act_scale, out, sums, err, s);
+    st = g.G >= TC_MIN_G ? launch_tc_contract(act, g, codes, alpha, act_scale, out, sums, err, s)
+         : sums          ? launch_tc4_sums(act, g, codes, sums, err, s)
+                         : launch_fold_contract(act, g, codes, alpha, act_scale, out, err, s);
   else
     st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
   if (a32 && cudaFreeAsync(a32, s) != cudaSuccess && st == FGQ_OK) st = FGQ_ERR_CUDA;
@@ -198,8 +211,6 @@ fgq_status after_launch(cudaError_t launch_result) {
 }
 
 int64_t debug_wait_limit_us() { return t_wait_limit_us; }
-
-bool debug_cta_pairs() { return t_cta_pairs != 0; }
 
 int debug_max_ksplit() { return t_max_ksplit; }
 

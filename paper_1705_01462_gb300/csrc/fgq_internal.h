@@ -37,8 +37,6 @@ fgq_status after_launch(cudaError_t launch_result);  // the result of a cudaLaun
 // Wait limit, in microseconds, that a test set on this host thread for the tensor-core
 // kernels' mbarrier waits (fgq_debug_set_wait_limit_us), or -1 for the kernels' own limits.
 int64_t debug_wait_limit_us();
-// Whether the G = 4 output kernel runs on CTA pairs (this thread's setting, default off).
-bool debug_cta_pairs();
 int debug_max_ksplit();    // 1 .. 8
 void note_ksplit(int k);   // group ranges of the G >= 64 tensor-core call just launched
 
@@ -78,12 +76,17 @@ fgq_status launch_tc_contract(const void* act, const Geom& g, const uint32_t* co
                               int32_t* sums, unsigned int* err, cudaStream_t s);
 
 
-// Tensor-core contraction for G = 4 (block-diagonal activation operand).
+// Tensor-core group sums for G = 4 (block-diagonal ternary operand): int32 [M][ng][P].
 bool tc4_supports(const Geom& g);
-// sums != nullptr writes the int32 group sums [M][ng][P] instead of the output.
-fgq_status launch_tc4_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
-                               const float* act_scale, float* out, int32_t* sums, unsigned int* err,
-                               cudaStream_t s);
+fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes, int32_t* sums, unsigned int* err,
+                           cudaStream_t s);
+
+// Tensor-core contraction for G in {4, 8, 16, 32}: the alphas folded into integer weights on a
+// common grid per 256 reduction elements, in two fp16 parts.  Any channel count, 8- or 4-bit
+// activations.
+bool fold_supports(const Geom& g);
+fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
+                                const float* act_scale, float* out, unsigned int* err, cudaStream_t s);
 
 // Dense tensor-core contraction with the alphas folded into fp16 weights: fixed-point alphas
 // (aq, abits 8 or 4, ascale) exactly, or fp32 alphas (aq == nullptr) split into two fp16
@@ -92,12 +95,6 @@ bool dense_supports(const Geom& g);
 fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
                                  const uint8_t* aq, int abits, const float* ascale, const float* act_scale, float* out,
                                  unsigned int* err, cudaStream_t s);
-// fp32 alphas folded into the codes as two fp16 parts: a0[m][k] + a1[m][k] = alpha(m, k / G) *
-// t[m][k] * 2^e_m to about 22 bits (a0 the fp16 nearest, a1 the fp16 nearest the remainder),
-// with e_m putting row m's largest alpha in [2^14, 2^15), and rs[m] = 2^-e_m.  a0, a1 fp16
-// [M][16 wrow]; codes 00 and padding give 0.
-fgq_status launch_fold_alpha_split(const uint32_t* codes, int M, int wrow, int G, int ng, const float* alpha,
-                                   void* a0, void* a1, float* rs, cudaStream_t s);
 // The 8-bit-weight convolution (dense weights wq, per-filter scales) on the same kernel, through
 // an explicit im2col of the activations in a pool temporary (any C, groups == 1); exact.
 bool dense_w8_supports(const Geom& g);

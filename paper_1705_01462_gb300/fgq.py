@@ -495,7 +495,7 @@ def fgq_debug_allow_split_fold(allow: bool) -> int:
 
 
 def fgq_debug_cta_pairs(on: bool) -> int:
-    """G = 4 output kernel on CTA pairs or single CTAs (the default) for this thread's calls."""
+    """Remembered only: every contraction kernel runs on single CTAs."""
     return int(lib().fgq_debug_cta_pairs(1 if on else 0))
 
 

@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
               fence_proxy_async_smem();
               __syncwarp();
               if (lane == 0) {
-                tma_store_2d(&a.out_map, m, pw + 32 * j, smem_u32(ob));
+                if (pw + 32 * j < g.P) tma_store_2d(&a.out_map, m, pw + 32 * j, smem_u32(ob));
                 bulk_commit();
               }
               if (++obuf == obufs) obuf = 0;

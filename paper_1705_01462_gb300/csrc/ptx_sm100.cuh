@@ -120,7 +120,7 @@ __device__ __forceinline__ bool mbar_wait_timed(uint64_t* bar, uint32_t parity, 
 // hardware only.
 __device__ __forceinline__ bool mbar_wait_quick(uint64_t* bar, uint32_t parity, uint64_t timeout_ns,
                                                 volatile uint32_t* abort) {
-  if (mbar_test_wait(bar, parity)) return true;
+  if (__builtin_expect(mbar_test_wait(bar, parity), 1)) return true;
   if (timeout_ns == 0) return false;
   if (mbar_try_wait_sleep(bar, parity, 1000u)) return true;
   const uint64_t t0 = globaltimer_ns();
@@ -130,6 +130,41 @@ __device__ __forceinline__ bool mbar_wait_quick(uint64_t* bar, uint32_t parity, 
   }
   return false;
 }
+
+// The same with the barrier's shared-memory address (loops that index their barriers keep 32-bit
+// addresses instead of generic pointers).
+__device__ __forceinline__ bool mbar_wait_quick(uint32_t bar, uint32_t parity, uint64_t timeout_ns,
+                                                volatile uint32_t* abort) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  if (__builtin_expect(ok, 1)) return true;
+  if (timeout_ns == 0) return false;
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t i = 0; i < (1u << 26); ++i) {
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(1000u)
+        : "memory");
+    if (ok) return true;
+    if ((i & 7u) == 7u && (*abort || globaltimer_ns() - t0 > timeout_ns)) return false;
+  }
+  return false;
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}" ::"r"(bar) : "memory");
+}
+
+// Registers of the calling warpgroup from now on (every warp of the warpgroup executes it): the
+// shares of a block's warpgroups must not add up to more than its launch's registers.
+template <int N>
+__device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
@@ -221,6 +256,17 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 registers into 16 consecutive columns of this thread's TMEM lane, and the wait for such stores
+// (before this thread reads them back).
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Waits for this thread's TMEM loads, with r as in/out operands so that no use of r is
 // placed before the wait (16-register form).

@@ -98,9 +98,16 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_have_cuda = False
+
+
 def _require_cuda():
+    global _have_cuda
+    if _have_cuda:
+        return
     if not torch.cuda.is_available():
         raise RuntimeError("libfgq needs a CUDA GPU; there is no CPU fallback")
+    _have_cuda = True
 
 
 def _check(code: int, what: str):
@@ -108,19 +115,28 @@ def _check(code: int, what: str):
         raise FGQError(code, what)
 
 
+# The raw handle of the current stream (0.1 us; torch.cuda.current_stream builds a Stream object
+# each time, 2.9 us a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _get_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_get_device())
 
 
 def _dev(t: torch.Tensor, dtype, name: str) -> int:
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous():
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    return t.data_ptr()
+    raise ValueError(f"{name} must be contiguous")
 
 
 def _act_type(t) -> int:
@@ -135,6 +151,17 @@ def codes_words_per_row(Kred: int, G: int) -> int:
 
 def num_groups(Kred: int, G: int) -> int:
     return int(lib().fgq_num_groups(Kred, G))
+
+
+_GROUP_SIZES = frozenset((1, 2, 4, 8, 16, 32, 64, 128))
+
+
+def _row_sizes(Kred: int, G: int) -> Tuple[int, int]:
+    """(code words, groups) per filter row; the library's own answer (0) for a bad G."""
+    if G in _GROUP_SIZES:
+        ng = (Kred + G - 1) // G
+        return (ng * G + 15) // 16, ng
+    return codes_words_per_row(Kred, G), num_groups(Kred, G)
 
 
 def quantize_act_workspace_bytes(n: int) -> int:
@@ -152,10 +179,11 @@ def fgq_ternarize(w: torch.Tensor, G: int, codes: Optional[torch.Tensor] = None,
     """w fp32 [M][Kred] -> (codes int32-view of uint32 [M][words], alpha fp32 [M][ng])."""
     _require_cuda()
     M, Kred = w.shape
+    words, ng = _row_sizes(Kred, G)
     if codes is None:
-        codes = torch.empty((M, codes_words_per_row(Kred, G)), dtype=torch.int32, device=w.device)
+        codes = torch.empty((M, words), dtype=torch.int32, device=w.device)
     if alpha is None:
-        alpha = torch.empty((M, num_groups(Kred, G)), dtype=torch.float32, device=w.device)
+        alpha = torch.empty((M, ng), dtype=torch.float32, device=w.device)
     _check(lib().fgq_ternarize(_dev(w, torch.float32, "w"), M, Kred, G, _dev(codes, torch.int32, "codes"),
                                _dev(alpha, torch.float32, "alpha"), _stream(stream)), "fgq_ternarize")
     return codes, alpha
@@ -169,18 +197,17 @@ def fgq_ternarize_batch(ws, G: int, stream=None):
     list of (codes, alpha)."""
     _require_cuda()
     n = len(ws)
-    outs = []
-    for w in ws:
-        M, Kred = w.shape
-        codes = torch.empty((M, codes_words_per_row(Kred, G)), dtype=torch.int32, device=w.device)
-        alpha = torch.empty((M, num_groups(Kred, G)), dtype=torch.float32, device=w.device)
-        outs.append((codes, alpha))
     VP, I = ctypes.c_void_p * max(n, 1), ctypes.c_int * max(n, 1)
-    tw = VP(*[_dev(w, torch.float32, "w") for w in ws])
-    tm = I(*[int(w.shape[0]) for w in ws])
-    tk = I(*[int(w.shape[1]) for w in ws])
-    tc = VP(*[c.data_ptr() for c, _ in outs])
-    ta = VP(*[a.data_ptr() for _, a in outs])
+    tw, tm, tk, tc, ta = VP(), I(), I(), VP(), VP()
+    outs = []
+    for i, w in enumerate(ws):
+        M, Kred = w.shape
+        words, ng = _row_sizes(Kred, G)
+        tw[i], tm[i], tk[i] = _dev(w, torch.float32, "w"), M, Kred
+        codes = torch.empty((M, words), dtype=torch.int32, device=w.device)
+        alpha = torch.empty((M, ng), dtype=torch.float32, device=w.device)
+        tc[i], ta[i] = codes.data_ptr(), alpha.data_ptr()
+        outs.append((codes, alpha))
     _check(lib().fgq_ternarize_batch(n, tw, tm, tk, G, tc, ta, _stream(stream)), "fgq_ternarize_batch")
     return outs
 

@@ -76,6 +76,14 @@ fgq_status launch_tc_contract(const void* act, const Geom& g, const uint32_t* co
                               int32_t* sums, unsigned int* err, cudaStream_t s);
 
 
+// The G >= 64 kernel as one dense contraction y = s_x rs[m] sum_k a16[m][k] q[p][k] on fp16 weights
+// [M][Kp] (K in (r, s, c) order, Cg % 64 == 0): x16 is scratch of tc_rows_act_bytes for the expanded
+// activations.  Products and sums of integers are exact below 2^24.
+bool tc_rows_supports(const Geom& g);
+size_t tc_rows_act_bytes(const Geom& g);
+fgq_status launch_tc_rows(const void* act, void* x16, const Geom& g, const void* a16, const float* rs,
+                          const float* act_scale, float* out, unsigned int* err, cudaStream_t s);
+
 // Tensor-core group sums for G = 4 (block-diagonal ternary operand): int32 [M][ng][P].
 bool tc4_supports(const Geom& g);
 fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes, int32_t* sums, unsigned int* err,

@@ -13,6 +13,10 @@
 //     carries about 22 bits of alpha; A0 = hi t, A1 = lo t, rs = 2^-e_m.  The accumulator
 //     rounds once per K = 16 step.
 //
+// This kernel converts 8-bit activations in flight.  Fixed-point alphas run on the dense form of the
+// G >= 64 kernel (an fp16 copy of the activations) wherever that is faster (reads_once below); split
+// fp32 alphas and im2col rows of 8-bit weights always run here.
+//
 // Tile: 128 filters x 256 positions, K-tile 64.  Each K-tile is 4 (or 8, two parts) MMAs
 // M = 128, N = 256, K = 16 into the tile's TMEM accumulator (256 columns); the epilogue runs
 // once per tile.  Two accumulators: the epilogue of tile i overlaps the MMAs of tile i + 1.
@@ -831,6 +835,21 @@ constexpr int64_t DENSE_W8_MAX_COL_BYTES = (int64_t)8 << 30;  // the im2col temp
 
 }  // namespace
 
+// Unpadded stride-1 1x1 layers and GEMMs of few filters and many rows: this kernel converts the 8-bit
+// rows in flight, the dense form of the G >= 64 kernel reads an fp16 copy (five bytes moved per
+// activation).  Measured, 8-bit alphas, this kernel against that form: 256 -> 64 on 56 x 56, batch 64,
+// 42 / 65 us; 64 -> 256 57 / 60; 512 -> 128 on 28 x 28 29 / 35; but 1024 -> 256 on 14 x 14 27 / 23;
+// 8192 rows of 1024 -> 1024 42 / 29; and where each activation is read at several taps always the
+// form: 3 x 3 at batch 64, 64 channels on 56 x 56 83 / 61, 256 on 14 x 14 59 / 25, 512 on 7 x 7 101 / 31.
+static bool reads_once(const Geom& g) {
+  if (g.R != 1 || g.S != 1 || g.stride != 1 || g.pad != 0 || g.M > 512) return false;
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t tiles = (int64_t)g.groups * ((g.Mg + TD_BM - 1) / TD_BM) * ((g.P + TD_BN - 1) / TD_BN);
+  return tiles >= 2 * sms || g.P * g.C >= (int64_t)16 << 20;
+}
+
 fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
                                  const uint8_t* aq, int abits, const float* ascale, const float* act_scale, float* out,
                                  unsigned int* err, cudaStream_t s) {
@@ -841,11 +860,14 @@ fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t*
   cudaMemPool_t pool = scratch_pool();
   if (!pool) return FGQ_ERR_CUDA;
   const size_t part_bytes = (size_t)g.M * g.Kp * 2;
+  const bool rows = NA == 1 && tc_rows_supports(g) && !reads_once(g);  // the dense form of the G >= 64 kernel
+  const size_t rs_off = NA * part_bytes, x_off = (rs_off + (size_t)g.M * 4 + 255) / 256 * 256;
   void* tmp = nullptr;
-  if (cudaMallocFromPoolAsync(&tmp, NA * part_bytes + (size_t)g.M * 4, pool, s) != cudaSuccess) return FGQ_ERR_CUDA;
+  if (cudaMallocFromPoolAsync(&tmp, x_off + (rows ? tc_rows_act_bytes(g) : 0), pool, s) != cudaSuccess)
+    return FGQ_ERR_CUDA;
   __half* a0 = static_cast<__half*>(tmp);
   __half* a1 = NA == 2 ? a0 + (size_t)g.M * g.Kp : nullptr;
-  float* rs = reinterpret_cast<float*>(static_cast<uint8_t*>(tmp) + NA * part_bytes);
+  float* rs = reinterpret_cast<float*>(static_cast<uint8_t*>(tmp) + rs_off);
   const unsigned fblocks = (unsigned)g.M;
   if (!aq)
     fold_weights_kernel<0><<<fblocks, FOLD_THREADS, 0, s>>>(codes, g.M, g.wrow, g.G, g.ng, alpha, nullptr, nullptr, a0,
@@ -857,7 +879,10 @@ fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t*
     fold_weights_kernel<4><<<fblocks, FOLD_THREADS, 0, s>>>(codes, g.M, g.wrow, g.G, g.ng, nullptr, aq, ascale, a0, a1,
                                                             rs);
   fgq_status st = after_launch();
-  if (st == FGQ_OK) st = run_dense(act, g, NA, a0, a1, rs, act_scale, out, err, s);
+  if (st == FGQ_OK && rows)
+    st = launch_tc_rows(act, static_cast<uint8_t*>(tmp) + x_off, g, a0, rs, act_scale, out, err, s);
+  else if (st == FGQ_OK)
+    st = run_dense(act, g, NA, a0, a1, rs, act_scale, out, err, s);
   // the temporary returns to the pool once the work queued on s before this point is done
   if (cudaFreeAsync(tmp, s) != cudaSuccess && st == FGQ_OK) st = FGQ_ERR_CUDA;
   return st;

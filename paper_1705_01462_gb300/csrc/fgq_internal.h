@@ -84,6 +84,12 @@ size_t tc_rows_act_bytes(const Geom& g);
 fgq_status launch_tc_rows(const void* act, void* x16, const Geom& g, const void* a16, const float* rs,
                           const float* act_scale, float* out, unsigned int* err, cudaStream_t s);
 
+// 8-bit-weight convolutions of few channels (at most 8, one conv group, at most 514 products per
+// output, so that every sum is exact) without im2col rows or any temporary.
+bool few_supports(const Geom& g);
+fgq_status launch_few(const void* act, const Geom& g, const int8_t* wq, const float* wscale, const float* act_scale,
+                      float* out, unsigned int* err, cudaStream_t s);
+
 // Tensor-core group sums for G = 4 (block-diagonal ternary operand): int32 [M][ng][P].
 bool tc4_supports(const Geom& g);
 fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes, int32_t* sums, unsigned int* err,

@@ -899,6 +899,7 @@ bool dense_w8_supports(const Geom& g) {
 fgq_status launch_dense_w8(const void* act, const Geom& g, const int8_t* wq, const float* wscale,
                            const float* act_scale, float* out, unsigned int* err, cudaStream_t s) {
   if (!dense_w8_supports(g)) return FGQ_ERR_UNSUPPORTED;
+  if (few_supports(g)) return launch_few(act, g, wq, wscale, act_scale, out, err, s);
   const int Kc = (g.Kred + TD_KT - 1) / TD_KT * TD_KT;
   cudaMemPool_t pool = scratch_pool();
   if (!pool) return FGQ_ERR_CUDA;

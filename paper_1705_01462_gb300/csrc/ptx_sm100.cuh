@@ -346,6 +346,20 @@ __device__ __forceinline__ uint64_t sdesc_k_sw64(uint32_t saddr) {
   return d;
 }
 
+// Rows of 32 bytes with the 32-byte swizzle: 8-row atoms of 256 B (stride byte offset 256).
+__device__ __forceinline__ uint64_t sdesc_k_sw32(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)(256 >> 4) << 32 |
+         (uint64_t)1 << 46 |  // descriptor version (sm_100 family)
+         (uint64_t)6 << 61;   // 32-byte swizzle
+}
+
+// A K-major tile without swizzle: core matrices of 8 rows x 16 bytes (rows 16 bytes apart), sbo bytes
+// from one group of 8 rows to the next, lbo bytes from one 16-byte piece of K to the next.
+__device__ __forceinline__ uint64_t sdesc_k_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(sbo >> 4) << 32 |
+         (uint64_t)1 << 46;  // descriptor version (sm_100 family)
+}
+
 // D[tmem] (+)= A[smem] * B[smem]^T with e4m3 A and B (kind::f8f6f4, K = 32 per MMA), fp32
 // accumulator.  The instruction descriptor is idesc_f16_f32's: format code 0 is e4m3 for this
 // kind.
@@ -402,6 +416,12 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, int c0, int c1, u
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
                    reinterpret_cast<uint64_t>(tmap)),
                "r"(c0), "r"(c1), "r"(src_smem)
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const void* tmap, int c0, int c1, int c2, uint32_t src_smem) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                   reinterpret_cast<uint64_t>(tmap)),
+               "r"(c0), "r"(c1), "r"(c2), "r"(src_smem)
                : "memory");
 }
 // Add a box from shared memory into global memory (fp32 elements of the map), element by

@@ -87,9 +87,12 @@ __global__ void __launch_bounds__(kThreads) qa_max_kernel(const float* __restric
 
 __device__ __forceinline__ int dfp_exponent(uint32_t mbits, int qmax) {
   if (mbits == 0 || mbits >= 0x7f800000u) return 0;
-  const double md = (double)__uint_as_float(mbits);
-  int E = (int)((__double_as_longlong(md) >> 52) & 0x7ff) - 1023 - 10;  // condition fails here
-  while (md * pow2d(-E) > (double)qmax) ++E;
+  // mbits = 1.f 2^e against qmax = 1.q 2^k: E = e - k, one more where 1.f exceeds 1.q (in fp64 every
+  // fp32 magnitude is normal)
+  const uint64_t b = (uint64_t)__double_as_longlong((double)__uint_as_float(mbits));
+  const uint64_t frac = ((uint64_t)1 << 52) - 1;
+  const int k = 31 - __clz(qmax);
+  const int E = (int)(b >> 52) - 1023 - k + ((b & frac) > (((uint64_t)qmax << (52 - k)) & frac) ? 1 : 0);
   return max(-149, min(127, E));
 }
 
@@ -99,6 +102,26 @@ template <> struct QTraits<FGQ_U8> { static constexpr int qmin = 0, qmax = 255, 
 template <> struct QTraits<FGQ_S8> { static constexpr int qmin = -128, qmax = 127, bits = 8; };
 template <> struct QTraits<FGQ_U4> { static constexpr int qmin = 0, qmax = 15, bits = 4; };
 template <> struct QTraits<FGQ_S4> { static constexpr int qmin = -8, qmax = 7, bits = 4; };
+
+// Four codes of an 8-bit type in a word: conversions, then saturating packs (the int32 conversion
+// saturates and takes NaN to 0, as in qcode).  ONE: mul2 is 1.
+template <int TYPE, bool ONE>
+__device__ __forceinline__ uint32_t qword(const float4& f, float mul1, float mul2) {
+  static_assert(QTraits<TYPE>::bits == 8, "8-bit codes");
+  const int a = __float2int_rn(ONE ? f.x * mul1 : f.x * mul1 * mul2);
+  const int b = __float2int_rn(ONE ? f.y * mul1 : f.y * mul1 * mul2);
+  const int c = __float2int_rn(ONE ? f.z * mul1 : f.z * mul1 * mul2);
+  const int d = __float2int_rn(ONE ? f.w * mul1 : f.w * mul1 * mul2);
+  uint32_t hi, r;
+  if (TYPE == FGQ_U8) {
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(d), "r"(c));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(b), "r"(a), "r"(hi));
+  } else {
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(d), "r"(c));
+    asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(b), "r"(a), "r"(hi));
+  }
+  return r;
+}
 
 template <int TYPE>
 __device__ __forceinline__ uint32_t qcode(float x, float mul1, float mul2) {
@@ -311,143 +334,166 @@ fgq_status launch_quantize(const float* x, size_t n, int type, int E_given, bool
 
 // ----------------------------------------------------------------------------------------
 // fgq_quantize_act_batch: the same quantization for many tensors (the inputs of a network's
-// layers), with far fewer launches.  The tensors are taken in order in chunks of at most
-// kBatchChunkBytes of fp32 input (a larger tensor forms a chunk of its own), so that what pass
-// 1 reads is still in the L2 when pass 2 re-reads it.  The passes are pipelined: launch k
-// quantizes chunk k - 1 (pass 2, from the L2) while it reduces chunk k (pass 1, from HBM),
-// so C chunks take C + 1 launches and the two passes overlap.  Every block covers
-// kBatchElems consecutive elements of one tensor.  Pass 1 folds its maximum into the
-// tensor's word with atomicMax (magnitude bit patterns order like the floats); pass 2 takes
-// the tensor's exponent from that word and quantizes its elements, blocks in reverse order
-// (the data pass 1 read last first).
+// layers) in one cooperative launch.  The tensors are cut into items of kBatchElems consecutive
+// elements, and taken in order in chunks of about kBatchChunkBytes of fp32 input.  The items of all
+// passes form one list -- pass 1 (the maximum) of chunk k, then pass 2 (the codes) of chunk k - 1 --
+// that the resident blocks work off in order, block b taking items b, b + grid, ...: pass 2 reads
+// from the L2 what pass 1 brought there shortly before, beside the HBM reads of the next chunk.
+//
+// A tensor's word holds its largest exponent so far, in an order-preserving code (the exponent of the
+// maximum is the maximum of the items' exponents), above the count of its items that pass 1 has
+// finished.  A pass 2 item waits until that count is complete; the items that it waits for precede it
+// in the list and wait for nothing, and all blocks are resident, so every wait ends (and is bounded
+// in time all the same: FGQ_ERR_TIMEOUT).
+//
+// Bound: one read of the inputs and one write of the codes (31 tensors, 162 M elements: 810 MB, 120
+// us).  That batch took 250 us as one launch per 48 MB chunk (15 launches of 17 us) and takes 199 a
+// call: 24 to 40 MB chunks, 64 or 128 KB items and 5 to 8 blocks per SM all give 195 to 200 (what is
+// left is the host's part of a call), items of 32 KB 226 (an item's maximum is then one batch of
+// loads, and a reduction and an atomic with nothing in flight).
 namespace fgq {
 namespace {
 
 constexpr int kBatchThreads = 256;
-constexpr int64_t kBatchElems = 16384;             // elements per block (64 KB of fp32)
-constexpr int kBatchChunk = 32;                    // tensors per launch
-constexpr size_t kBatchChunkBytes = (size_t)48 << 20;  // two chunks (one per pass) share the L2
+constexpr int kBatchBlocks = 5;                        // resident blocks per SM
+constexpr int kBatchElems = 16384;                     // elements per item (64 KB of fp32)
+constexpr size_t kBatchChunkBytes = (size_t)24 << 20;  // two chunks and their codes stay in the L2
+constexpr int kBatchCountBits = 23;                    // of a tensor's word; its exponent code above
+constexpr uint32_t kBatchBadCode = 511;                // a NaN or infinity: exponent 0, and above all others
+constexpr uint64_t kBatchTimeoutNs = 2000000000ull;
 
 struct QTensor {
   const float* x;
   uint8_t* q;
   float* scale;
-  unsigned int* tmax;  // the tensor's maximum word
+  unsigned int* word;
   int64_t n;
   int type;
-  int block0;   // first block of this tensor in the launch
+  int items;
 };
 
+// Items first, first + 1, ... (up to the next segment's first): pass 1 or 2 of one tensor.
+struct QSegment {
+  int first;
+  int16_t tensor;
+  int16_t pass;
+};
+
+template <int MAXT>
 struct QBatch {
-  QTensor t[kBatchChunk];
-  int n;
-  int nblocks;
+  QTensor t[MAXT];
+  QSegment seg[2 * MAXT];
+  int nseg;
+  int items;
 };
 
-__device__ __forceinline__ int qbatch_tensor(const QBatch& b, int blk) {
-  int lo = 0, hi = b.n - 1;
-  while (lo < hi) {  // largest tensor whose first block is <= blk
-    const int mid = (lo + hi + 1) >> 1;
-    if (b.t[mid].block0 <= blk) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+__device__ __forceinline__ uint32_t exponent_code(uint32_t mbits, int qmax) {
+  return mbits == 0 ? 0u : (mbits >= 0x7f800000u ? kBatchBadCode : (uint32_t)(dfp_exponent(mbits, qmax) + 150));
+}
+__device__ __forceinline__ int code_exponent(uint32_t code) {
+  return code == 0 || code == kBatchBadCode ? 0 : (int)code - 150;
+}
+__device__ __forceinline__ uint32_t load_acquire(const unsigned int* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
-__device__ __forceinline__ void qab_max_block(const QBatch& b, int blk, unsigned int* err) {
-  const QTensor& T = b.t[qbatch_tensor(b, blk)];
-  const int64_t e0 = (int64_t)(blk - T.block0) * kBatchElems;
+__device__ __forceinline__ void qab_max_item(const QTensor& T, int item, uint32_t* red, unsigned int* err) {
+  const int64_t e0 = (int64_t)item * kBatchElems;
   const int64_t e1 = e0 + kBatchElems < T.n ? e0 + kBatchElems : T.n;
   const bool is_unsigned = T.type == FGQ_U8 || T.type == FGQ_U4;
-  uint32_t mx = 0;
-  bool bad = false;
+  // mag: the largest magnitude pattern (NaN and infinities above all finite ones); pos: the largest
+  // pattern as a signed integer, so that negative floats count as 0 for the unsigned types
+  uint32_t mag = 0;
+  int pos = 0;
+  auto take = [&](float e) {
+    mag = max(mag, __float_as_uint(e) & 0x7fffffffu);
+    pos = max(pos, __float_as_int(e));
+  };
   const float4* x4 = reinterpret_cast<const float4*>(T.x + e0);  // e0 is a multiple of 4: aligned
-  const int64_t n4 = (e1 - e0) / 4;
+  const int n4 = (int)((e1 - e0) / 4);
   const uint64_t keep = policy_evict_last();
   constexpr int U = 8;  // independent 16-byte loads in flight per thread
-  int64_t i = threadIdx.x;
+  int i = threadIdx.x;
   for (; i + (U - 1) * kBatchThreads < n4; i += U * kBatchThreads) {
     float4 f[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) f[u] = ld_f4_policy(x4 + i + u * kBatchThreads, keep);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const float e[4] = {f[u].x, f[u].y, f[u].z, f[u].w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        bad |= (__float_as_uint(e[j]) & 0x7fffffffu) >= 0x7f800000u;
-        mx = max(mx, mag_bits(e[j], is_unsigned));
-      }
+      take(f[u].x);
+      take(f[u].y);
+      take(f[u].z);
+      take(f[u].w);
     }
   }
   for (; i < n4; i += kBatchThreads) {
     const float4 f = ld_f4_policy(x4 + i, keep);
-    const float e[4] = {f.x, f.y, f.z, f.w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      bad |= (__float_as_uint(e[j]) & 0x7fffffffu) >= 0x7f800000u;
-      mx = max(mx, mag_bits(e[j], is_unsigned));
-    }
+    take(f.x);
+    take(f.y);
+    take(f.z);
+    take(f.w);
   }
-  for (int64_t i = e0 + n4 * 4 + threadIdx.x; i < e1; i += kBatchThreads) {
-    const float e = __ldg(T.x + i);
-    bad |= (__float_as_uint(e) & 0x7fffffffu) >= 0x7f800000u;
-    mx = max(mx, mag_bits(e, is_unsigned));
-  }
-  __shared__ uint32_t red[kBatchThreads / 32];
+  for (int64_t j = e0 + (int64_t)n4 * 4 + threadIdx.x; j < e1; j += kBatchThreads) take(__ldg(T.x + j));
+  uint32_t mx = is_unsigned ? (uint32_t)pos : mag;
+  const bool bad = mag >= 0x7f800000u;
   mx = __reduce_max_sync(FULL_MASK, mx);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   if (__syncthreads_or(bad) && threadIdx.x == 0) record_error(err, FGQ_ERR_NONFINITE);
   if (threadIdx.x == 0) {
     uint32_t m = 0;
     for (int i = 0; i < kBatchThreads / 32; ++i) m = max(m, red[i]);
-    atomicMax(T.tmax, m);
+    const int qmax = T.type == FGQ_U8 ? 255 : (T.type == FGQ_S8 ? 127 : (T.type == FGQ_U4 ? 15 : 7));
+    const uint32_t code = exponent_code(m, qmax);
+    uint32_t w = *reinterpret_cast<volatile unsigned int*>(T.word);
+    while (code > w >> kBatchCountBits) {  // raise the exponent and count in one step
+      const uint32_t old = atomicCAS(T.word, w, (code << kBatchCountBits) | ((w & ((1u << kBatchCountBits) - 1u)) + 1u));
+      if (old == w) return;
+      w = old;
+    }
+    atomicAdd(T.word, 1u);  // (a word's exponent never falls)
   }
 }
 
-template <int TYPE>
-__device__ __forceinline__ void qab_quant_range(const QTensor& T, int64_t e0, int64_t e1, bool write_scale) {
+// Four consecutive codes per thread and step: a warp loads 512 consecutive bytes and stores 128 (or 64).
+template <int TYPE, bool ONE>
+__device__ __forceinline__ void qab_quant_quads(const float4* x4, uint8_t* q, int n4, float mul1, float mul2) {
   using Tr = QTraits<TYPE>;
-  const int E = dfp_exponent(*reinterpret_cast<const volatile unsigned int*>(T.tmax), Tr::qmax);
+  const uint64_t drop = policy_evict_first();
+  auto put = [&](int i, const float4& f) {
+    if constexpr (Tr::bits == 8)
+      reinterpret_cast<uint32_t*>(q)[i] = qword<TYPE, ONE>(f, mul1, mul2);
+    else
+      reinterpret_cast<uint16_t*>(q)[i] =
+          (uint16_t)(qcode<TYPE>(f.x, mul1, mul2) | (qcode<TYPE>(f.y, mul1, mul2) << 4) |
+                     (qcode<TYPE>(f.z, mul1, mul2) << 8) | (qcode<TYPE>(f.w, mul1, mul2) << 12));
+  };
+  constexpr int U = 8;
+  int i = threadIdx.x;
+  for (; i + (U - 1) * kBatchThreads < n4; i += U * kBatchThreads) {
+    float4 f[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) f[u] = ld_f4_policy(x4 + i + u * kBatchThreads, drop);
+#pragma unroll
+    for (int u = 0; u < U; ++u) put(i + u * kBatchThreads, f[u]);
+  }
+  for (; i < n4; i += kBatchThreads) put(i, ld_f4_policy(x4 + i, drop));
+}
+
+template <int TYPE>
+__device__ __forceinline__ void qab_quant_range(const QTensor& T, int64_t e0, int64_t e1, bool write_scale, int E) {
+  using Tr = QTraits<TYPE>;
   if (write_scale && threadIdx.x == 0) *T.scale = pow2f(E);
   const float mul1 = (-E <= 127) ? pow2f(-E) : pow2f(64);
   const float mul2 = (-E <= 127) ? 1.0f : pow2f(-E - 64);
-  const int64_t n16 = (e1 - e0) / 16;
+  const int n4 = (int)((e1 - e0) / 4);
   const float4* x4 = reinterpret_cast<const float4*>(T.x + e0);
-  const uint64_t drop = policy_evict_first();
-  constexpr int CU = 2;  // 16-element chunks in flight per thread (8 independent 16-byte loads)
-  for (int64_t c0 = threadIdx.x; c0 < n16; c0 += CU * kBatchThreads) {
-    float e[CU][16];
-#pragma unroll
-    for (int u = 0; u < CU; ++u) {
-      const int64_t c = c0 + u * kBatchThreads;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float4 f = c < n16 ? ld_f4_policy(x4 + 4 * c + j, drop) : make_float4(0.f, 0.f, 0.f, 0.f);
-        e[u][4 * j] = f.x; e[u][4 * j + 1] = f.y; e[u][4 * j + 2] = f.z; e[u][4 * j + 3] = f.w;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < CU; ++u) {
-      const int64_t c = c0 + u * kBatchThreads;
-      if (c >= n16) break;
-      if (Tr::bits == 8) {
-        uint32_t wv[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          wv[j] = qcode<TYPE>(e[u][4 * j], mul1, mul2) | (qcode<TYPE>(e[u][4 * j + 1], mul1, mul2) << 8) |
-                  (qcode<TYPE>(e[u][4 * j + 2], mul1, mul2) << 16) | (qcode<TYPE>(e[u][4 * j + 3], mul1, mul2) << 24);
-        reinterpret_cast<uint4*>(T.q + e0)[c] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-      } else {
-        uint32_t wv[2] = {0u, 0u};
-#pragma unroll
-        for (int j = 0; j < 16; ++j) wv[j / 8] |= qcode<TYPE>(e[u][j], mul1, mul2) << (4 * (j % 8));
-        reinterpret_cast<uint2*>(T.q + e0 / 2)[c] = make_uint2(wv[0], wv[1]);
-      }
-    }
-  }
-  if (threadIdx.x == 0) {  // the tensor's ragged tail (last block only): fewer than 16 elements
-    for (int64_t i = e0 + n16 * 16; i < e1; ++i) {
+  uint8_t* q = T.q + (Tr::bits == 8 ? e0 : e0 / 2);
+  if (-E <= 127) qab_quant_quads<TYPE, true>(x4, q, n4, mul1, mul2);
+  else qab_quant_quads<TYPE, false>(x4, q, n4, mul1, mul2);
+  if (threadIdx.x == 0) {  // the tensor's ragged tail (last block only): fewer than 4 elements
+    for (int64_t i = e0 + (int64_t)n4 * 4; i < e1; ++i) {
       const uint32_t code = qcode<TYPE>(T.x[i], mul1, mul2);
       if (Tr::bits == 8) {
         T.q[i] = (uint8_t)code;
@@ -460,31 +506,120 @@ __device__ __forceinline__ void qab_quant_range(const QTensor& T, int64_t e0, in
   }
 }
 
-__device__ __forceinline__ void qab_quant_block(const QBatch& b, int blk) {
-  const QTensor& T = b.t[qbatch_tensor(b, blk)];
-  const int64_t e0 = (int64_t)(blk - T.block0) * kBatchElems;
+__device__ __forceinline__ void qab_quant_item(const QTensor& T, int item, int E) {
+  const int64_t e0 = (int64_t)item * kBatchElems;
   const int64_t e1 = e0 + kBatchElems < T.n ? e0 + kBatchElems : T.n;
-  const bool first = blk == T.block0;
   switch (T.type) {
-    case FGQ_U8: qab_quant_range<FGQ_U8>(T, e0, e1, first); break;
-    case FGQ_S8: qab_quant_range<FGQ_S8>(T, e0, e1, first); break;
-    case FGQ_U4: qab_quant_range<FGQ_U4>(T, e0, e1, first); break;
-    default: qab_quant_range<FGQ_S4>(T, e0, e1, first); break;
+    case FGQ_U8: qab_quant_range<FGQ_U8>(T, e0, e1, item == 0, E); break;
+    case FGQ_S8: qab_quant_range<FGQ_S8>(T, e0, e1, item == 0, E); break;
+    case FGQ_U4: qab_quant_range<FGQ_U4>(T, e0, e1, item == 0, E); break;
+    default: qab_quant_range<FGQ_S4>(T, e0, e1, item == 0, E); break;
   }
 }
 
-// One pipelined launch: blocks [0, q.nblocks) quantize chunk q (reverse block order), the
-// rest reduce chunk m.
-struct QPair {
-  QBatch q, m;
-};
+template <int MAXT>
+__global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) qab_kernel(const __grid_constant__ QBatch<MAXT> p,
+                                                                        unsigned int* err) {
+  __shared__ uint32_t red[2][kBatchThreads / 32];  // alternating: an item's is read while the next is reduced
+  __shared__ int sE[2];
+  int b = 0, cur = -1, E = 0;
+  for (int i = blockIdx.x; i < p.items; i += gridDim.x) {
+    int lo = 0, hi = p.nseg - 1;
+    while (lo < hi) {  // the last segment that starts at or before i
+      const int mid = (lo + hi + 1) >> 1;
+      if (p.seg[mid].first <= i) lo = mid;
+      else hi = mid - 1;
+    }
+    const QTensor& T = p.t[p.seg[lo].tensor];
+    const int item = i - p.seg[lo].first;
+    if (p.seg[lo].pass == 1) {
+      qab_max_item(T, item, red[b], err);
+      b ^= 1;
+    } else {
+      if (p.seg[lo].tensor != cur) {  // the same tensor as before: its exponent is known
+        bool late = false;
+        if (threadIdx.x == 0) {
+          const uint32_t mask = (1u << kBatchCountBits) - 1u;
+          uint32_t w;
+          uint64_t t0 = 0;
+          while (((w = load_acquire(T.word)) & mask) != (uint32_t)T.items) {
+            uint64_t now;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kBatchTimeoutNs) {
+              record_error(err, FGQ_ERR_TIMEOUT);
+              late = true;
+              break;
+            }
+            __nanosleep(100);
+          }
+          sE[b] = code_exponent(w >> kBatchCountBits);
+        }
+        if (__syncthreads_or(late)) return;
+        E = sE[b];
+        b ^= 1;
+        cur = p.seg[lo].tensor;
+      }
+      qab_quant_item(T, item, E);
+    }
+  }
+}
 
-__global__ void __launch_bounds__(kBatchThreads) qab_kernel(const __grid_constant__ QPair p, unsigned int* err) {
-  pdl_wait();  // the previous launch's maxima (and the zeroed words) are complete
-  pdl_trigger();
-  const int bx = (int)blockIdx.x;
-  if (bx < p.q.nblocks) qab_quant_block(p.q, p.q.nblocks - 1 - bx);
-  else qab_max_block(p.m, bx - p.q.nblocks, err);
+template <int MAXT>
+fgq_status launch_qab(int n, const float* const* x, const size_t* nelem, const int* type, void* const* q,
+                      float* const* scale_out, unsigned int* words, unsigned int* err, cudaStream_t s) {
+  QBatch<MAXT> p;
+  memset(&p, 0, sizeof p);
+  int nt = 0;
+  for (int i = 0; i < n; ++i) {
+    if (nelem[i] == 0) continue;
+    const int64_t items = ((int64_t)nelem[i] + kBatchElems - 1) / kBatchElems;
+    if (items >= (int64_t)1 << kBatchCountBits) return FGQ_ERR_UNSUPPORTED;  // 256 GB of input
+    QTensor& T = p.t[nt++];
+    T.x = x[i];
+    T.q = static_cast<uint8_t*>(q[i]);
+    T.scale = scale_out[i];
+    T.word = words + i;
+    T.n = (int64_t)nelem[i];
+    T.type = type[i];
+    T.items = (int)items;
+  }
+  if (nt == 0) return FGQ_OK;
+  int64_t total = 0;
+  auto add = [&](int t0, int t1, int pass) {
+    for (int t = t0; t < t1; ++t) {
+      p.seg[p.nseg].first = (int)total;
+      p.seg[p.nseg].tensor = (int16_t)t;
+      p.seg[p.nseg++].pass = (int16_t)pass;
+      total += p.t[t].items;
+    }
+  };
+  int prev = 0;  // first tensor of the chunk that waits for pass 2
+  for (int t = 0; t < nt;) {
+    // a chunk: consecutive tensors up to kBatchChunkBytes of input (at least one tensor)
+    int end = t;
+    size_t bytes = 0;
+    while (end < nt && (end == t || bytes + (size_t)p.t[end].n * sizeof(float) <= kBatchChunkBytes))
+      bytes += (size_t)p.t[end++].n * sizeof(float);
+    add(t, end, 1);
+    add(prev, t, 2);
+    prev = t;
+    t = end;
+  }
+  add(prev, nt, 2);
+  if (total > INT32_MAX / 2) return FGQ_ERR_UNSUPPORTED;
+  p.items = (int)total;
+  const int64_t cap = (int64_t)num_sms() * kBatchBlocks;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(total < cap ? total : cap));
+  cfg.blockDim = dim3(kBatchThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return after_launch(cudaLaunchKernelEx(&cfg, qab_kernel<MAXT>, p, err));
 }
 
 }  // namespace
@@ -492,56 +627,10 @@ __global__ void __launch_bounds__(kBatchThreads) qab_kernel(const __grid_constan
 size_t quantize_batch_workspace_bytes(int n) { return n > 0 ? sizeof(unsigned int) * (size_t)n : 0; }
 
 fgq_status launch_quantize_batch(int n, const float* const* x, const size_t* nelem, const int* type, void* const* q,
-                                 float* const* scale_out, unsigned int* tmax, unsigned int* err, cudaStream_t s) {
-  if (cudaMemsetAsync(tmax, 0, sizeof(unsigned int) * (size_t)n, s) != cudaSuccess) return FGQ_ERR_CUDA;
-  QPair p;
-  memset(&p, 0, sizeof p);  // p.q: the chunk waiting for pass 2 (none yet)
-  int i = 0;
-  auto launch = [&]() -> fgq_status {
-    const int64_t blocks = (int64_t)p.q.nblocks + p.m.nblocks;
-    if (blocks == 0) return FGQ_OK;
-    if (blocks > INT32_MAX) return FGQ_ERR_UNSUPPORTED;
-    return after_launch(launch_pdl(qab_kernel, dim3((unsigned)blocks), dim3(kBatchThreads), 0, s, p, err));
-  };
-  while (i < n) {
-    QBatch& b = p.m;
-    memset(&b, 0, sizeof b);
-    size_t bytes = 0;
-    int blocks = 0;
-    // a chunk: consecutive tensors up to kBatchChunkBytes of input (at least one tensor)
-    while (i < n && b.n < kBatchChunk) {
-      if (nelem[i] == 0) {
-        ++i;
-        continue;
-      }
-      const size_t tb = nelem[i] * sizeof(float);
-      if (b.n > 0 && bytes + tb > kBatchChunkBytes) break;
-      const int64_t nb = ((int64_t)nelem[i] + kBatchElems - 1) / kBatchElems;
-      if ((int64_t)blocks + nb > INT32_MAX) {
-        if (b.n == 0) return FGQ_ERR_UNSUPPORTED;  // one tensor beyond the grid's reach
-        break;
-      }
-      QTensor& T = b.t[b.n++];
-      T.x = x[i];
-      T.q = static_cast<uint8_t*>(q[i]);
-      T.scale = scale_out[i];
-      T.tmax = tmax + i;
-      T.n = (int64_t)nelem[i];
-      T.type = type[i];
-      T.block0 = blocks;
-      blocks += (int)nb;
-      bytes += tb;
-      ++i;
-    }
-    if (b.n == 0) continue;
-    b.nblocks = blocks;
-    // pass 2 of the previous chunk and pass 1 of this one
-    const fgq_status st = launch();
-    if (st != FGQ_OK) return st;
-    p.q = p.m;
-  }
-  memset(&p.m, 0, sizeof p.m);
-  return launch();  // pass 2 of the last chunk
+                                 float* const* scale_out, unsigned int* words, unsigned int* err, cudaStream_t s) {
+  if (cudaMemsetAsync(words, 0, sizeof(unsigned int) * (size_t)n, s) != cudaSuccess) return FGQ_ERR_CUDA;
+  return n <= 32 ? launch_qab<32>(n, x, nelem, type, q, scale_out, words, err, s)
+                 : launch_qab<FGQ_QUANTIZE_BATCH_MAX>(n, x, nelem, type, q, scale_out, words, err, s);
 }
 
 }  // namespace fgq

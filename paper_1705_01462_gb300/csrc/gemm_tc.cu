@@ -24,7 +24,7 @@
 //
 // Warp roles (384 threads, one CTA per SM, persistent over tiles):
 //   warps 0-7  epilogue: warp w reads TMEM lanes 32*(w%4).. (filter rows) and the positions of half
-//              w/4 of the drained buffer in 64-column tcgen05.ld, adds alpha * s into 128 fp32
+//              w/4 of the drained buffer in 32-column tcgen05.ld, adds alpha * s into 128 fp32
 //              registers and frees the buffer.  At tile end it stores boxes of 16 positions x 32
 //              filters through its own buffers by TMA (or directly), requantized when asked.
 //              The drain bounds this kernel: about 1040 clk per group of 256 positions against 512 of
@@ -94,14 +94,10 @@ static_assert(TC_SMEM <= 232448, "shared memory budget");
 // activations, F8): every 4-bit value and every code is exact in e4m3, so the K-tile is
 // 64-byte rows with the 64-byte swizzle and 2 MMAs of K = 32 (kind::f8f6f4) -- half the bytes
 // per K-tile in HBM, L2 and shared memory, twice the ring depth.
-// Activation boxes of a K-tile: an im2col box (the tile's output positions at one filter tap and
-// 64 channels, padding read as zeros), or a 2D box where the positions are input rows.
-enum { ACT_IM2COL = 0, ACT_2D = 1 };
-
 template <bool F8>
 struct TcCfg {
-  static constexpr int ROW = TC_KT * (F8 ? 1 : 2);  // bytes per operand row of a K-tile
-  static constexpr int A_TILE = TC_BM * ROW;        // weight operand; the activations take bn rows
+  static constexpr int ES = F8 ? 1 : 2;              // bytes per operand element
+  static constexpr int A_TILE = TC_BM * TC_KT * ES;  // ternary operand; the activations take bn * 64 * ES
 };
 
 struct TcArgs {
@@ -121,7 +117,7 @@ struct TcArgs {
   int ksplit;       // group ranges per tile (1: whole tiles; > 1: partial sums added into the output)
   int gpk;          // groups per range
   int kt_per_group; // G / 64
-  int act_mode;     // how the activations are loaded (ACT_*)
+  int act_tma;      // 2D activation map (one row per output position); else im2col map
   int out_tma;      // output boxes by TMA store
   int bn, nst;      // positions per tile, ring depth
   int nacc;         // TMEM accumulator buffers of bn columns
@@ -129,26 +125,21 @@ struct TcArgs {
   uint64_t timeout_ns;
 };
 
-// Work item w: tile w / ksplit, groups [g0, g1) of range w % ksplit, output positions from p0.  Tiles are numbered with the filter tiles of one position tile consecutive, so that CTAs running
-// at the same time share activation boxes in L2.
-struct Item {
-  int gi, m0, g0, g1;
-  int64_t p0;
-};
-__device__ __forceinline__ Item item_coords(const TcArgs& a, int w) {
-  Item it;
+// Work item w: tile w / ksplit, groups [g0, g1) of range w % ksplit.  Tiles are numbered
+// with the filter tiles of one position tile consecutive, so that CTAs running at the same
+// time share activation boxes in L2.
+__device__ __forceinline__ void item_coords(const TcArgs& a, int w, int& gi, int& m0, int64_t& p0, int& g0, int& g1) {
   const int tile = w / a.ksplit;
   const int ks = w - tile * a.ksplit;
   const int per_p = a.g.groups * a.mtiles;
   const int pt = tile / per_p;
   const int r = tile - pt * per_p;
-  it.gi = r / a.mtiles;
-  const int mt = r - it.gi * a.mtiles;
-  it.m0 = it.gi * a.g.Mg + mt * TC_BM;
-  it.p0 = (int64_t)pt * a.bn;
-  it.g0 = ks * a.gpk;
-  it.g1 = it.g0 + a.gpk < a.g.ng ? it.g0 + a.gpk : a.g.ng;
-  return it;
+  gi = r / a.mtiles;
+  const int mt = r - gi * a.mtiles;
+  m0 = gi * a.g.Mg + mt * TC_BM;
+  p0 = (int64_t)pt * a.bn;
+  g0 = ks * a.gpk;
+  g1 = g0 + a.gpk < a.g.ng ? g0 + a.gpk : a.g.ng;
 }
 
 // One launch prepares both operands of a call: blocks [0, code_blocks) expand the ternary codes
@@ -181,11 +172,14 @@ __global__ void __launch_bounds__(256) prep64_kernel(const uint32_t* __restrict_
   }
 }
 
-// OUT: 0 fp32, 1 requantized codes, 2
+// TMAP: the layer's im2col rows are contiguous input rows (2D box loads); otherwise the
+// activation boxes come from an im2col map (one load per K-tile: the tile's output positions at
+// one filter tap and 64 channels, padding read as zeros).  OUT: 0 fp32, 1 requantized codes, 2
 // int32 group sums (kernels of their own, so that each epilogue's unrolled code stays short).
-template <int ACT, int OUT, bool F8>
+template <bool TMAP, int OUT, bool F8>
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid_constant__ TcArgs a) {
-  constexpr int ROW = TcCfg<F8>::ROW, A_TILE = TcCfg<F8>::A_TILE;
+  constexpr int ES = TcCfg<F8>::ES;
+  constexpr int A_TILE = TcCfg<F8>::A_TILE;
   constexpr bool SUMS = OUT == 2, RQ = OUT == 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -203,7 +197,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
   const Geom& g = a.g;
   const uint64_t tmo = a.timeout_ns;
   const int nst = a.nst, nacc = a.nacc;
-  const uint32_t stage = (uint32_t)(A_TILE + a.bn * ROW);
+  const uint32_t stage = (uint32_t)(A_TILE + a.bn * TC_KT * ES);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < nst; ++i) {
@@ -247,10 +241,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
       uint32_t ph = 1;  // parity of the stage's previous release; the first round passes at once
       bool ok = true;
       for (int tl = 0; tl < my_tiles && ok; ++tl) {
-        const Item it = item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x);
+        int gi, m0, g0, g1;
+        int64_t p0;
+        item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x, gi, m0, p0, g0, g1);
         int n0 = 0, h0 = 0, w0 = 0;  // im2col: the tile's first window origin (input pixel coordinates)
-        if (ACT == ACT_IM2COL) {
-          const int pp = (int)it.p0;  // < P < 2^31
+        if (!TMAP) {
+          const int pp = (int)p0;  // < P < 2^31
           const int wo = pp % g.Wo;
           const int q = pp / g.Wo;
           n0 = q / g.Ho;
@@ -259,9 +255,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
         }
         // the range's first K-tile and its filter tap (tr, ts) and channel offset tc0, which
         // then advance incrementally
-        const int kt0 = it.g0 * a.kt_per_group, kt1 = it.g1 * a.kt_per_group;
+        const int kt0 = g0 * a.kt_per_group, kt1 = g1 * a.kt_per_group;
         int tc0 = (kt0 % kpt) * TC_KT, ts = (kt0 / kpt) % g.S, tr = (kt0 / kpt) / g.S;
-        const int cb = it.gi * g.Cg;  // a multiple of 64 (128-byte aligned in fp16)
+        const int cb = gi * g.Cg;  // a multiple of 64 (128-byte aligned in fp16)
         for (int kt = kt0; kt < kt1; ++kt) {
           if (!mbar_wait_quick(&empty[s], ph, tmo, abort_flag)) {
             ok = false;
@@ -270,9 +266,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
           if (elect_one()) {
             const uint32_t sa = sbase + (uint32_t)s * stage;
             mbar_arrive_expect_tx(&full[s], stage);
-            tma_load_2d(sa, &a.a16_map, kt * TC_KT, it.m0, &full[s]);
-            if (ACT == ACT_2D)
-              tma_load_2d(sa + A_TILE, &a.act_map, cb + tc0, (int)it.p0, &full[s]);
+            tma_load_2d(sa, &a.a16_map, kt * TC_KT, m0, &full[s]);
+            if (TMAP)
+              tma_load_2d(sa + A_TILE, &a.act_map, cb + tc0, (int)p0, &full[s]);
             else
               tma_load_im2col_4d(sa + A_TILE, &a.act_map, cb + tc0, w0, h0, n0, (uint16_t)ts, (uint16_t)tr, &full[s]);
           }
@@ -301,14 +297,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
       // ---------------------------------------------------------------- MMA issuers
       const int b = warp - TC_MMA_WARP;  // parity of the groups this warp issues
       const uint32_t idesc = idesc_f16_f32(TC_BM, a.bn);
-      const uint64_t ad0 = ROW == 64 ? sdesc_k_sw64(smem_u32(smem)) : sdesc_k_sw128(smem_u32(smem));
-      const uint64_t bd0 = ROW == 64 ? sdesc_k_sw64(smem_u32(smem) + A_TILE) : sdesc_k_sw128(smem_u32(smem) + A_TILE);
+      const uint64_t ad0 = F8 ? sdesc_k_sw64(smem_u32(smem)) : sdesc_k_sw128(smem_u32(smem));
+      const uint64_t bd0 = F8 ? sdesc_k_sw64(smem_u32(smem) + A_TILE) : sdesc_k_sw128(smem_u32(smem) + A_TILE);
       int s = 0, gc = 0, ab = 0;  // ring position, group count, accumulator of group gc
       uint32_t ph = 0, aph = 1;
       bool ok = true;
       for (int tl = 0; tl < my_tiles && ok; ++tl) {
-        const Item it = item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x);
-        for (int grp = it.g0; grp < it.g1 && ok; ++grp, ++gc) {
+        int gi_, m0_, g0, g1;
+        int64_t p0_;
+        item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x, gi_, m0_, p0_, g0, g1);
+        for (int grp = g0; grp < g1 && ok; ++grp, ++gc) {
           const bool mine = (gc & 1) == b;
           if (mine && !mbar_wait_quick(&acc_empty[ab], aph, tmo, abort_flag)) {
             ok = false;
@@ -373,12 +371,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
     uint32_t fph = 0;
     bool ok = true;
     for (int tl = 0; tl < my_tiles; ++tl) {
-      const Item it = item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x);
-      const int g0 = it.g0, g1 = it.g1, m0 = it.m0;
+      int gi, m0, g0, g1;
+      int64_t p0;
+      item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x, gi, m0, p0, g0, g1);
       const int m = m0 + t;
-      const int mend = it.gi * g.Mg + g.Mg;  // the conv group's filters end here
+      const int mend = gi * g.Mg + g.Mg;  // the conv group's filters end here
       const bool mok = m < mend;
-      const int64_t pbase = it.p0 + hcols * part;
+      const int64_t pbase = p0 + hcols * part;
       const float* acol = SUMS ? nullptr : a.alpha_t + (int64_t)g0 * g.M + (mok ? m : 0);
       float acc[TC_EPI_COLS];
       if (!SUMS) {
@@ -451,7 +450,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
         uint32_t v[16];
         tmem_ld16(ta + 16 * c, v);
         tmem_ld_wait_regs16(v);
-        const int pb = (int)pbase + 16 * c;
         if (a.out_tma) {
           // a box of 16 positions x 32 filters through the warp's own buffers; positions past P and
           // filters past M are clipped by the tensor map
@@ -470,6 +468,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
+            const int pb = (int)pbase + 16 * c;
             if (wok && pb < g.P) {
               if (!RQ && a.ksplit > 1)  // a group range's partial sums: added into the (zeroed) output
                 tma_reduce_add_2d(&a.out_map, m, pb, smem_u32(ob));
@@ -483,7 +482,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
           // the warp's 32 lanes are 32 consecutive filters
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int64_t p = pb + j;
+            const int64_t p = pbase + 16 * c + j;
             if (p < g.P) {
               const float y = sx * __uint_as_float(v[j]);
               if (RQ) g.rq_out[p * g.M + m] = rq_code(y, rq);
@@ -512,18 +511,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
   }
 }
 
-template <int ACT, int OUT, bool F8>
+template <bool TMAP, int OUT, bool F8>
 fgq_status launch_tc(const TcArgs& args, int grid, cudaStream_t s) {
-  if (!tc::smem_attr_once<tc_contract_kernel<ACT, OUT, F8>>(TC_SMEM)) return FGQ_ERR_CUDA;
-  return after_launch(launch_pdl(tc_contract_kernel<ACT, OUT, F8>, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, args));
+  if (!tc::smem_attr_once<tc_contract_kernel<TMAP, OUT, F8>>(TC_SMEM)) return FGQ_ERR_CUDA;
+  return after_launch(launch_pdl(tc_contract_kernel<TMAP, OUT, F8>, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, args));
 }
 
 template <bool F8>
 fgq_status launch_tc_variant(const TcArgs& a, int grid, cudaStream_t s) {
-  const bool rows = a.act_mode == ACT_2D;
-  if (a.sums) return rows ? launch_tc<ACT_2D, 2, F8>(a, grid, s) : launch_tc<ACT_IM2COL, 2, F8>(a, grid, s);
-  if (a.g.rq_out) return rows ? launch_tc<ACT_2D, 1, F8>(a, grid, s) : launch_tc<ACT_IM2COL, 1, F8>(a, grid, s);
-  return rows ? launch_tc<ACT_2D, 0, F8>(a, grid, s) : launch_tc<ACT_IM2COL, 0, F8>(a, grid, s);
+  if (a.sums) return a.act_tma ? launch_tc<true, 2, F8>(a, grid, s) : launch_tc<false, 2, F8>(a, grid, s);
+  if (a.g.rq_out) return a.act_tma ? launch_tc<true, 1, F8>(a, grid, s) : launch_tc<false, 1, F8>(a, grid, s);
+  return a.act_tma ? launch_tc<true, 0, F8>(a, grid, s) : launch_tc<false, 0, F8>(a, grid, s);
 }
 
 // One block waits on an mbarrier that nothing arrives on; every wait is bounded, so the
@@ -701,12 +699,12 @@ fgq_status launch_tc_contract(const void* act, const Geom& g, const uint32_t* co
   if (st == FGQ_OK && !make_map_2d(&a.a16_map, dt, a16, (uint64_t)g.wrow * 16, (uint64_t)g.M,
                                    (uint64_t)g.wrow * 16 * es, TC_KT, TC_BM, sw))
     st = FGQ_ERR_CUDA;
-  a.act_mode = act_pointwise(g) ? ACT_2D : ACT_IM2COL;
+  a.act_tma = act_pointwise(g) ? 1 : 0;
   bool act_ok = true;
   if (st == FGQ_OK) {
     if (!f8)
       act_ok = tc::act16_map(&a.act_map, x16, g, (uint32_t)a.bn);
-    else if (a.act_mode == ACT_2D)
+    else if (a.act_tma)
       act_ok = make_map_2d(&a.act_map, dt, x16, (uint64_t)g.C, (uint64_t)(nact / g.C), (uint64_t)g.C, TC_KT,
                            (uint32_t)a.bn, sw);
     else
@@ -767,7 +765,7 @@ fgq_status launch_tc_rows(const void* act, void* x16, const Geom& g, const void*
                    TC_KT, TC_BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !tc::act16_map(&a.act_map, x16, g, (uint32_t)a.bn))
     return FGQ_ERR_CUDA;
-  a.act_mode = act_pointwise(g) ? ACT_2D : ACT_IM2COL;
+  a.act_tma = act_pointwise(g) ? 1 : 0;
   plan_out_map(a, out);
   return launch_tc_variant<false>(a, a.ntiles < sms ? a.ntiles : sms, s);
 }

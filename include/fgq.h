@@ -253,7 +253,7 @@ fgq_status fgq_quantize_weights_w8(const float* w, int M, int Kred, int8_t* wq, 
  * stream-ordered pool of the current device and return them on the same stream: the
  * activations as fp16 (2 bytes per element read; for G < 64 each conv group's channels padded
  * to a multiple of 64), and the ternary operand -- at G >= 64 the codes as fp16 (2 * M * Kp
- * bytes), for G < 64 the folded weights (two fp16 parts, and room for the parts that widely
+ * bytes) and the alphas transposed (4 * M * ng bytes), for G < 64 the folded weights (two fp16 parts, and room for the parts that widely
  * spread alphas need: 8 * M' * Kp' bytes, M' and Kp' padded to multiples of 64; the group sums
  * of G = 4 take 8 * M' * Kp bytes for a block-diagonal form instead).
  * The pool keeps freed blocks, so only a call that needs more than the pool holds reaches
@@ -357,7 +357,8 @@ fgq_status fgq_quantize_alpha(const float* alpha, int M, int ng, int bits, uint8
  * exactly in 64-bit integers: y = act_scale * ascale[m] * sum, rounded once.  Otherwise, with
  * 8-bit activations and Cg a multiple of 64, the automatic choice is the dense tensor-core
  * path (FGQ_PATH_DENSE): the integer weights aq * t are folded into an fp16 matrix in a pool
- * temporary (2 * M * Kp bytes) and one dense contraction sums the exact integer products in
+ * temporary (2 * M * Kp bytes; beside it, where activations are read more than once, an fp16
+ * copy of them) and one dense contraction sums the exact integer products in
  * an fp32 accumulator: y = act_scale * ascale[m] * sum is the exact value rounded once when
  * sum_k |aq t q| < 2^24 (which bounds every partial sum; e.g. always for Kred * 255 * 255 <
  * 2^24), and otherwise within (Kp / 16) * 2^-23 * act_scale * ascale[m] * sum_k |aq t q| of it

@@ -70,19 +70,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
-// Waits (sleeping in the hardware for up to sleep_ns per poll) for the phase with the given
-// parity; gives up after max_iter polls or once *abort becomes non-zero, so that one
-// role's timeout releases the roles waiting on it.  max_iter polls bound the wait by
-// max_iter * sleep_ns (plus the hardware's own short limit per poll).
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, uint32_t max_iter,
-                                                   volatile uint32_t* abort, uint32_t sleep_ns = 20000u) {
-  for (uint32_t i = 0; i < max_iter; ++i) {
-    if (mbar_try_wait_sleep(bar, parity, sleep_ns)) return true;
-    if (*abort) return false;
-  }
-  return false;
-}
-
 // Nanoseconds of the GPU's global timer.
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
@@ -267,7 +254,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
       : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Waits for this thread's TMEM loads, with r as in/out operands so that no use of r is
 // placed before the wait (16-register form).
 __device__ __forceinline__ void tmem_ld_wait_regs16(uint32_t (&r)[16]) {

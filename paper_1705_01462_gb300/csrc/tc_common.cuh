@@ -37,48 +37,6 @@ __device__ __forceinline__ uint32_t u8pair_to_h2(uint32_t x, uint32_t sel, uint3
   return r;
 }
 
-// Expansion of 2-bit codes: a nibble (two codes) -> two fp16 {0, +1, -1}, stored 32 times
-// ([16][32] words) so that lane l reads copy l and no two lanes share a bank.
-__device__ __forceinline__ void fill_code_lut(uint32_t* lut) {
-  for (int i = threadIdx.x; i < 16 * 32; i += blockDim.x) {
-    const uint32_t x = (uint32_t)i >> 5;
-    uint32_t h[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const uint32_t c = (x >> (2 * e)) & 3u;
-      h[e] = c == 1u ? 0x3C00u : (c == 3u ? 0xBC00u : 0u);
-    }
-    lut[i] = h[0] | (h[1] << 16);
-  }
-}
-
-// Converts the 64 codes (16 bytes) of one K-tile row to fp16 into row t of a 128B-swizzled
-// K-major operand tile; lut = the table above, offset by the calling lane.
-__device__ __forceinline__ void codes_row_to_fp16(const uint8_t* codes16, uint8_t* tile, int t, const uint32_t* lt) {
-  uint32_t cw[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) cw[i] = *reinterpret_cast<const uint32_t*>(codes16 + 4 * i);
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const uint32_t bits = (cw[c / 2] >> (16 * (c & 1))) & 0xffffu;  // 8 codes
-    *reinterpret_cast<uint4*>(tile + sw128(t, c)) =
-        make_uint4(lt[32 * (bits & 15u)], lt[32 * ((bits >> 4) & 15u)], lt[32 * ((bits >> 8) & 15u)], lt[32 * (bits >> 12)]);
-  }
-}
-
-// Half h (codes 32 h .. 32 h + 31, 8 bytes) of one K-tile row: 16-byte chunks 4 h .. 4 h + 3
-// of row t of the 128B-swizzled operand tile.
-__device__ __forceinline__ void codes_half_row_to_fp16(const uint8_t* codes16, int h, uint8_t* tile, int t,
-                                                       const uint32_t* lt) {
-  const uint2 cw = *reinterpret_cast<const uint2*>(codes16 + 8 * h);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t bits = ((i < 2 ? cw.x : cw.y) >> (16 * (i & 1))) & 0xffffu;  // 8 codes
-    *reinterpret_cast<uint4*>(tile + sw128(t, 4 * h + i)) =
-        make_uint4(lt[32 * (bits & 15u)], lt[32 * ((bits >> 4) & 15u)], lt[32 * ((bits >> 8) & 15u)], lt[32 * (bits >> 12)]);
-  }
-}
-
 // Raises a kernel's dynamic shared-memory limit to `bytes`, once per device (the attribute
 // belongs to the device's context); thread-safe.  Returns false if the call failed.
 template <auto Kernel>

@@ -71,7 +71,10 @@ bool tc_any(const Geom& g) { return g.G == 4 ? tc4_supports(g) : tc_supports(g);
 
 bool gemv_any(const Geom& g) { return !g.is_conv && gemv_supports((int)g.P, g.Kred, g.G, g.act_type); }
 
-// Layers with G < 64 that the automatic choice leaves to the dp4a kernel: fewer filters or
+// Layers that the folded kernel takes: G < 64, or G = 64 where the per-group kernel does not fit and
+// there are enough groups for its error to be the smaller one
+// (channels that are no multiple of 64: 5x5 with 2 x 48 channels on 27 x 27, batch 256, G = 64, dp4a
+// 1742 us a call, folded 205).  Left to the dp4a kernel: fewer filters or
 // channels per conv group than fill a 64 x 64 weight image by a fair part, and layers so small
 // that dp4a, which needs no operand preparation, is done first -- its time is about 0.05 us per
 // reduction element and wave of 64 x 128 output blocks (two blocks per SM), against two launches:
@@ -84,6 +87,10 @@ constexpr int TC_MIN_G = 64;  // from here on a group fills an MMA K-tile
 
 bool fold_any(const Geom& g) {
   if (g.Mg < FOLD_MIN_FILTERS || g.Cg < FOLD_MIN_CHANNELS || !fold_supports(g)) return false;
+  if (g.G >= TC_MIN_G) {
+    const int units = (g.R * g.S * ((g.Cg + 63) / 64) + 3) / 4;  // fp32 adds of the folded kernel
+    if (g.ng < FOLD_FEW_GROUPS || 2 * g.ng < 5 * units) return false;
+  }
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -112,7 +119,7 @@ int choose_path(const Geom& g, bool sums, bool qa) {
   // fixed-point alphas fold exactly into fp16 weights: one dense tensor-core contraction
   if (qa && dense_supports(g)) return FGQ_PATH_DENSE;
   // automatic choice: the tensor cores where the shape is covered
-  return (g.G < TC_MIN_G ? fold_any(g) : tc_any(g)) ? FGQ_PATH_TC : FGQ_PATH_SIMT;
+  return (g.G >= TC_MIN_G && tc_any(g)) || fold_any(g) ? FGQ_PATH_TC : FGQ_PATH_SIMT;
 }
 
 // Fixed-point alphas of a contraction call (nullptr: fp32 alphas).
@@ -151,7 +158,7 @@ fgq_status contract(const void* act, const Geom& g, const uint32_t* codes, const
   }
   fgq_status st;
   if (path == FGQ_PATH_TC)
-    st = g.G >= TC_MIN_G ? launch_tc_contract(act, g, codes, alpha, act_scale, out, sums, err, s)
+    st = g.G >= TC_MIN_G && tc_supports(g) ? launch_tc_contract(act, g, codes, alpha, act_scale, out, sums, err, s)
          : sums          ? launch_tc4_sums(act, g, codes, sums, err, s)
                          : launch_fold_contract(act, g, codes, alpha, act_scale, out, err, s);
   else

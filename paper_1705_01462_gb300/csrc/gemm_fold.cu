@@ -1,5 +1,6 @@
 // Tensor-core (tcgen05) grouped ternary contraction with the group scales folded into the
-// weights, for groups smaller than an MMA K-tile (G = 4, 8, 16, 32).
+// weights, for groups smaller than an MMA K-tile (G = 4, 8, 16, 32) and for G = 64 where the channels
+// do not fill the K-tiles of the per-group kernel.
 //
 // Eq. 2 is one dense contraction, y[p][m] = s_x sum_k A[m][k] q[p][k] with A = alpha(m, k / G)
 // t[m][k], if it can be summed without losing what the 32-bit group accumulators of Section 4
@@ -18,7 +19,9 @@
 // filter of the tile holds a non-zero alpha with v < 16 (more than 64 times below the row's
 // largest) gets a third part, fp16 of what (hi, lo) leave out times 2^24, contracted in a pass
 // of its own over the unit: then every alpha is carried to 22 bits or more.  The preparation
-// marks such units (about 1 in 300 for Gaussian weights at G = 4, rarer for larger G).
+// marks such units (about 1 in 300 for Gaussian weights at G = 4, rarer for larger G), and at G >= 8
+// all units of layers with few groups (FOLD_FEW_GROUPS), whose few fp32 adds err less than two
+// parts of the alphas would.
 //
 // hi and lo are two rows of the same MMA operand: a tile is 64 filters x up to 256 positions,
 // 128 operand rows (rows 32 q + i and 32 q + 16 + i: hi and lo of filter 16 q + i), so that one
@@ -135,6 +138,7 @@ struct PrepFold {
   uint8_t* ext;
   int wrow, ng, gshift;  // G = 1 << gshift
   int Mg, Cg, cpad, mtiles, ktiles, nunits, nsub, fold_blocks;
+  int third;             // every unit carries the third part
   int quads;             // Cg % 4 == 0: 4 elements from a multiple of 4 lie in one tap and one group
   int padded;            // activations need the padded expansion
   int fast8;             // ... of 8-bit codes in aligned runs of 8 (Cg and C multiples of 8)
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
       if (lane + 32 * j < PF_GPU) al[fl][lane + 32 * j] = v[i][j] * mul;  // exact: a power-of-two scaling
     if (sub == 0 && lane == 0) f.rs[((int64_t)tile * f.nunits + u) * TF_FM + fl] = pow2f(-e);
   }
-  const bool ext = __syncthreads_or(small);
+  const bool ext = __syncthreads_or(small) || f.third;
   if (sub == 0 && threadIdx.x == 0) f.ext[(int64_t)tile * f.nunits + u] = ext ? 1 : 0;
 
   // 16-byte chunks of the images: chunk c (8 elements) of the operand rows of filter fl
@@ -723,7 +727,7 @@ int choose_bn(int64_t P, int wtiles, int ktiles, int sms) {
 }  // namespace
 
 bool fold_supports(const Geom& g) {
-  if (g.G != 4 && g.G != 8 && g.G != 16 && g.G != 32) return false;
+  if (g.G < 4 || g.G > 64 || (g.G & (g.G - 1)) != 0) return false;
   if (g.P >= (int64_t)1 << 31) return false;  // positions decoded in 32 bits
   if (tc::encode_tiled() == nullptr) return false;
   return tc::act_pointwise(g) || (tc::encode_im2col() != nullptr && tc::im2col_fits(g.R, g.S, g.stride, g.pad));
@@ -790,6 +794,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.ktiles = a.ktiles;
   f.nunits = a.nunits;
   f.nsub = wtiles * a.nunits >= 2 * sms ? 1 : TF_UNIT;
+  f.third = g.G > 4 && g.ng < FOLD_FEW_GROUPS ? 1 : 0;
   f.quads = g.Cg % 4 == 0 ? 1 : 0;
   f.padded = (a.cpad != g.Cg || g.C % 16 != 0) ? 1 : 0;
   f.fast8 = f.padded && g.Cg % 8 == 0 && g.C % 8 == 0 && (g.act_type == FGQ_U8 || g.act_type == FGQ_S8) ? 1 : 0;

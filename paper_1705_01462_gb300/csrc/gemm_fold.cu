@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
   const int k0 = tap0 * f.Cg + (c0 < f.Cg ? c0 : f.Cg), k1 = tap1 * f.Cg + (c1 < f.Cg ? c1 : f.Cg);
   const int g0 = k0 >> f.gshift, g1 = ((k1 - 1) >> f.gshift) + 1;  // k1 > k0: a K-tile holds real channels
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  bool small = false;
+  bool small = f.third != 0;
   float v[TF_FM / 8][3];  // 8 filters per warp, every load in flight at once
 #pragma unroll
   for (int i = 0; i < TF_FM / 8; ++i) {
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
       if (lane + 32 * j < PF_GPU) al[fl][lane + 32 * j] = v[i][j] * mul;  // exact: a power-of-two scaling
     if (sub == 0 && lane == 0) f.rs[((int64_t)tile * f.nunits + u) * TF_FM + fl] = pow2f(-e);
   }
-  const bool ext = __syncthreads_or(small) || f.third;
+  const bool ext = __syncthreads_or(small);
   if (sub == 0 && threadIdx.x == 0) f.ext[(int64_t)tile * f.nunits + u] = ext ? 1 : 0;
 
   // 16-byte chunks of the images: chunk c (8 elements) of the operand rows of filter fl

@@ -94,6 +94,15 @@ int fgq_debug_max_ksplit(int k);
 int fgq_debug_last_ksplit(void);
 
 /*
+ * Self test of the wait that the warps of the tensor-core kernels share: the lanes of one warp wait,
+ * for at most limit_us microseconds, on phases of which half are complete and half never will be.
+ * Records FGQ_ERR_TIMEOUT if the wait expired for every lane, as it must (lanes that part here would
+ * part ahead of warp-collective instructions), FGQ_ERR_UNSUPPORTED otherwise; read the result with
+ * fgq_stream_status().
+ */
+fgq_status fgq_debug_selftest_warp_wait(uint32_t limit_us, cudaStream_t stream);
+
+/*
  * The CUDA runtime error (a cudaError_t value) behind the last FGQ_ERR_CUDA that a kernel
  * launch of this thread returned, 0 if none; reading it clears it.  `name` receives the
  * runtime's name of that error (at most `len` bytes including the terminator) when non-null.

@@ -744,4 +744,8 @@ fgq_status fgq_selftest_wait_timeout(uint32_t max_iterations, cudaStream_t strea
   return launch_wait_timeout_selftest(max_iterations, device_error_word(), stream);
 }
 
+fgq_status fgq_debug_selftest_warp_wait(uint32_t limit_us, cudaStream_t stream) {
+  return launch_wait_warp_selftest((uint64_t)limit_us * 1000u, device_error_word(), stream);
+}
+
 }  // extern "C"

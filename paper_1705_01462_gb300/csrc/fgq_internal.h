@@ -125,6 +125,7 @@ fgq_status launch_dense_w8(const void* act, const Geom& g, const int8_t* wq, con
                            const float* act_scale, float* out, unsigned int* err, cudaStream_t s);
 
 fgq_status launch_wait_timeout_selftest(uint32_t max_iter, unsigned int* err, cudaStream_t s);
+fgq_status launch_wait_warp_selftest(uint64_t limit_ns, unsigned int* err, cudaStream_t s);
 
 // Chained-forward steps: max pooling of u8 codes, residual addition of two 8-bit code
 // tensors (fp32 sum, or requantized when out_q is given).

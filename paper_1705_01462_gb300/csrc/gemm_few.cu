@@ -171,11 +171,11 @@ __global__ void __launch_bounds__(FW_THREADS, 1) few_kernel(const __grid_constan
     const uint64_t ad0 = sdesc_k_sw32(smem_u32(smem));
     const uint32_t ablk = (uint32_t)a.arows * 32u >> 4;
     const uint32_t rowb = (uint32_t)a.pitch * 16u;
-    bool ok = my_tiles <= 0 || mbar_wait_quick(a_full, 0, tmo, abort_flag);
+    bool ok = my_tiles <= 0 || mbar_wait_warp(a_full, 0, tmo, abort_flag);
     for (int tl = 0; tl < my_tiles && ok; ++tl) {
       const int s = tl & 1;
       const uint32_t ph = (uint32_t)(tl >> 1) & 1u;
-      if (!mbar_wait_quick(&acc_empty[s], ph ^ 1u, tmo, abort_flag) || !mbar_wait_quick(&full[s], ph, tmo, abort_flag)) {
+      if (!mbar_wait_warp(&acc_empty[s], ph ^ 1u, tmo, abort_flag) || !mbar_wait_warp(&full[s], ph, tmo, abort_flag)) {
         ok = false;
         break;
       }
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) few_kernel(const __grid_constan
           }
         }
         if (!free) {
-          ok = mbar_wait_quick(&empty[s], ((uint32_t)(tl >> 1) & 1u) ^ 1u, tmo, abort_flag);
+          ok = mbar_wait_warp(&empty[s], ((uint32_t)(tl >> 1) & 1u) ^ 1u, tmo, abort_flag);
           free = true;
           if (!ok) break;
         }
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1) few_kernel(const __grid_constan
     bool ok = true;
     for (int tl = 0; tl < my_tiles; ++tl) {
       const int s = tl & 1;
-      if (!mbar_wait_quick(&acc_full[s], (uint32_t)(tl >> 1) & 1u, tmo, abort_flag)) {
+      if (!mbar_wait_warp(&acc_full[s], (uint32_t)(tl >> 1) & 1u, tmo, abort_flag)) {
         ok = false;
         break;
       }

@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
           ts = uts;
           tc0 = utc;
           for (int j = 0; j < nk; ++j, asrc += TF_A) {
-            if (!mbar_wait_quick(&empty[s], ph, tmo, abort_flag)) {
+            if (!mbar_wait_warp(&empty[s], ph, tmo, abort_flag)) {
               ok = false;
               break;
             }
@@ -525,14 +525,14 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
             for (s += nk; s >= nst; s -= nst) ph ^= 1u;
             continue;
           }
-          if (!mbar_wait_quick(&acc_empty[b], aph, tmo, abort_flag) || !mbar_wait_quick(&turn[b], tph, tmo, abort_flag)) {
+          if (!mbar_wait_warp(&acc_empty[b], aph, tmo, abort_flag) || !mbar_wait_warp(&turn[b], tph, tmo, abort_flag)) {
             ok = false;
             break;
           }
           aph ^= 1u;
           tph ^= 1u;
           for (int j = 0; j < nk; ++j) {
-            if (!mbar_wait_quick(&full[s], ph, tmo, abort_flag)) {
+            if (!mbar_wait_warp(&full[s], ph, tmo, abort_flag)) {
               ok = false;
               break;
             }
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
         for (int pass = 0; pass < passes; ++pass) {
           if (!ok) continue;  // after a failed wait: run out the tile, then leave with the others
           const float r = pass ? r0 * 0x1p-24f : r0;  // the third part (in hi's rows) carries 2^24
-          if (!mbar_wait_quick(&acc_full[b], fph, tmo, abort_flag)) {
+          if (!mbar_wait_warp(&acc_full[b], fph, tmo, abort_flag)) {
             ok = false;
             continue;
           }

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
         int tc0 = (kt0 % kpt) * TC_KT, ts = (kt0 / kpt) % g.S, tr = (kt0 / kpt) / g.S;
         const int cb = gi * g.Cg;  // a multiple of 64 (128-byte aligned in fp16)
         for (int kt = kt0; kt < kt1; ++kt) {
-          if (!mbar_wait_quick(&empty[s], ph, tmo, abort_flag)) {
+          if (!mbar_wait_warp(&empty[s], ph, tmo, abort_flag)) {
             ok = false;
             break;
           }
@@ -308,13 +308,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
         item_coords(a, (int)blockIdx.x + tl * (int)gridDim.x, gi_, m0_, p0_, g0, g1);
         for (int grp = g0; grp < g1 && ok; ++grp, ++gc) {
           const bool mine = (gc & 1) == b;
-          if (mine && !mbar_wait_quick(&acc_empty[ab], aph, tmo, abort_flag)) {
+          if (mine && !mbar_wait_warp(&acc_empty[ab], aph, tmo, abort_flag)) {
             ok = false;
             break;
           }
           const uint32_t d = tmem + (uint32_t)(ab * a.bn);
           for (int sub = 0; sub < a.kt_per_group; ++sub) {
-            if (!mbar_wait_quick(&full[s], ph, tmo, abort_flag)) {
+            if (!mbar_wait_warp(&full[s], ph, tmo, abort_flag)) {
               ok = false;
               break;
             }
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_contract_kernel(const __grid
       for (int grp = g0; grp < g1; ++grp) {
         const float al = al_next;  // alpha of this group, loaded one group ahead
         if (!SUMS && grp + 1 < g1) al_next = __ldg(acol += g.M);
-        if (!mbar_wait_quick(bar_full + 8u * (uint32_t)b, fph, tmo, abort_flag)) {
+        if (!mbar_wait_warp(bar_full + 8u * (uint32_t)b, fph, tmo, abort_flag)) {
           ok = false;  // leave with the others below
           break;
         }
@@ -535,6 +535,22 @@ __global__ void wait_timeout_selftest_kernel(uint32_t max_iter, unsigned int* er
   __syncthreads();
   const bool ok = mbar_wait_bounded(&bar, 0, max_iter);
   if (!ok && threadIdx.x == 0) record_error(err, FGQ_ERR_TIMEOUT);
+}
+
+// One warp waits on one barrier for two phases at once: the even lanes' phase is complete, the odd
+// lanes' never will be.  A wait that the lanes decide together expires for all of them.
+__global__ void wait_warp_selftest_kernel(uint64_t limit_ns, unsigned int* err) {
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ uint32_t abort_flag;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    abort_flag = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const bool ok = mbar_wait_warp(&bar, (threadIdx.x & 1) ^ 1, limit_ns, &abort_flag);
+  const uint32_t passed = __ballot_sync(0xffffffffu, ok);
+  if (threadIdx.x == 0) record_error(err, passed == 0 ? FGQ_ERR_TIMEOUT : FGQ_ERR_UNSUPPORTED);
 }
 
 }  // namespace
@@ -772,6 +788,11 @@ fgq_status launch_tc_rows(const void* act, void* x16, const Geom& g, const void*
 
 fgq_status launch_wait_timeout_selftest(uint32_t max_iter, unsigned int* err, cudaStream_t s) {
   wait_timeout_selftest_kernel<<<1, 32, 0, s>>>(max_iter, err);
+  return after_launch();
+}
+
+fgq_status launch_wait_warp_selftest(uint64_t limit_ns, unsigned int* err, cudaStream_t s) {
+  wait_warp_selftest_kernel<<<1, 32, 0, s>>>(limit_ns, err);
   return after_launch();
 }
 

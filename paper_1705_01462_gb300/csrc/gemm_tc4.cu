@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(T4_THREADS, 1) tc4_sums_kernel(const __grid_co
       for (int k = 0; k < units_per_tile; ++k, ++u) {
         if (!ok) continue;
         const int b = u & 1;
-        if (!mbar_wait_timed(&acc_full[b], (u >> 1) & 1, tmo, abort_flag, 0)) {
+        if (!mbar_wait_warp(&acc_full[b], (u >> 1) & 1, tmo, abort_flag)) {
           ok = false;
           continue;
         }

@@ -64,6 +64,7 @@ SIGNATURES = [
     ("fgq_selftest_wait_timeout", _i, [_u32, _vp]),
     ("fgq_debug_set_wait_limit_us", _i64, [_i64]),
     ("fgq_debug_allow_split_fold", _i, [_i]),
+    ("fgq_debug_selftest_warp_wait", _i, [_u32, _vp]),
     ("fgq_debug_last_cuda_error", _i, [_vp, _sz]),
     ("fgq_debug_cta_pairs", _i, [_i]),
     ("fgq_debug_max_ksplit", _i, [_i]),
@@ -553,4 +554,9 @@ def fgq_launch_count() -> int:
 
 def fgq_selftest_wait_timeout(max_iterations: int, stream=None) -> int:
     _check(lib().fgq_selftest_wait_timeout(max_iterations, _stream(stream)), "fgq_selftest_wait_timeout")
+    return fgq_stream_status(stream)
+
+
+def fgq_debug_selftest_warp_wait(limit_us: int, stream=None) -> int:
+    _check(lib().fgq_debug_selftest_warp_wait(limit_us, _stream(stream)), "fgq_debug_selftest_warp_wait")
     return fgq_stream_status(stream)

@@ -79,3 +79,36 @@ def test_forced_wait_expiry_then_exact(family, G, R):
         out = call().cpu().numpy()
         assert fgq.fgq_stream_status() == fgq.FGQ_OK
         check_within(out, y, ym, f"{family} after an expired call")
+
+
+@pytest.mark.parametrize("limit_us", [0, 1, 200])
+def test_warp_wait_is_decided_once(limit_us):
+    """The lanes of a warp leave a wait together, also where some of them see their phase complete and
+    others run out of time: what follows a wait in the kernels are warp-collective instructions."""
+    assert fgq.fgq_debug_selftest_warp_wait(limit_us) == fgq.FGQ_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("family,G,R", [("tc4", 4, 3), ("tc", 64, 3), ("tc", 64, 1)])
+@pytest.mark.parametrize("limit_us", [1, 5])
+def test_short_wait_limits(family, G, R, limit_us):
+    """Limits near the waits' own lengths, so that the timer decides: some calls expire and some do not,
+    those that do not are right, and so is the next call with the normal limits."""
+    rng = np.random.default_rng(57 + G + R)
+    B, H, W, C, M = 8, 14, 14, 256, 256
+    t, al, codes = make_codes(rng.standard_normal((M, R * R * C)).astype(np.float32), G)
+    q, sc, packed = quantize_oracle(random_acts((B, H, W, C), "u8", rng), "u8")
+    y, ym = O.conv2d(q, sc, R, R, 1, R // 2, 1, t, al, G)
+    args = (to_dev(packed), "u8", to_dev(np.array([sc], np.float32)), B, H, W, C, R, R, 1, R // 2, 1,
+            to_dev(codes.view(np.int32)), to_dev(al), M, G)
+    fgq.fgq_set_path(fgq.PATH_TC)
+    fgq.fgq_debug_set_wait_limit_us(limit_us)
+    for _ in range(TRIES):
+        out = fgq.fgq_conv2d(*args)
+        st = fgq.fgq_stream_status()
+        assert st in (fgq.FGQ_OK, fgq.FGQ_ERR_TIMEOUT), st
+        if st == fgq.FGQ_OK:
+            check_within(out.cpu().numpy(), y, ym, f"{family} limit {limit_us} us")
+    fgq.fgq_debug_set_wait_limit_us(-1)
+    out = fgq.fgq_conv2d(*args).cpu().numpy()
+    assert fgq.fgq_stream_status() == fgq.FGQ_OK
+    check_within(out, y, ym, f"{family} after short limits")

@@ -5,8 +5,8 @@
 // Eq. 2 is one dense contraction, y[p][m] = s_x sum_k A[m][k] q[p][k] with A = alpha(m, k / G)
 // t[m][k], if it can be summed without losing what the 32-bit group accumulators of Section 4
 // keep.  Here it can, because the folded weights are integers on a common grid: the reduction
-// is cut into units of 256 elements, and in each unit row m is scaled by a power of two 2^e that
-// puts its largest alpha into (2^10, 2^11]; with v = alpha 2^e,
+// is cut into units of about 256 elements and whole groups (plan_units), and in each unit row m is
+// scaled by a power of two 2^e that puts its largest alpha into (2^10, 2^11]; with v = alpha 2^e,
 //     hi = rint(v),   lo = fp16((v - hi) 2^12),
 // both exact in fp16 (hi an integer of magnitude <= 2048).  Products hi t q are integers below
 // 2^19, so a unit's sum over 256 of them is the exact integer as long as it stays below 2^24 --
@@ -72,7 +72,8 @@ using tc::make_map_im2col;
 constexpr int TF_ROWS = 128;      // MMA M
 constexpr int TF_FM = 64;         // filters per tile (two operand rows each)
 constexpr int TF_KT = 64;         // reduction elements per K-tile: 4 MMAs
-constexpr int TF_UNIT = 4;        // K-tiles per unit (one TMEM accumulation)
+constexpr int TF_UNIT = 4;        // K-tiles per unit (one TMEM accumulation) where its groups allow it,
+constexpr int TF_MAX_UNIT = 8;    // and at most (plan_units)
 constexpr int TF_MAX_BN = 256;    // positions per tile (MMA N), a multiple of 64
 constexpr int TF_MAX_NST = 8;     // operand ring depth, at most (as many stages as fit)
 constexpr int TF_EPI_WARPS = 8;
@@ -100,7 +101,7 @@ static_assert(TF_SMEM <= 232448, "shared memory budget");
 struct FoldArgs {
   CUtensorMap act_map;   // fp16 activations: 2D [positions][Ca] or im2col, box 64 channels x bn positions
   CUtensorMap out_map;   // out_tma: outputs [P][M] (fp32 or codes), box {16 filters, 32 positions}
-  const uint8_t* a_op;   // weight K-tile images [tile][ktiles] of TF_A bytes
+  const uint8_t* a_op;   // weight K-tile images [tile][nunits][uk + ux] of TF_A bytes
   const uint8_t* a_ext;  // the third parts, same layout (written where ext is set)
   const float* rs;       // 2^-e [tile][nunits][TF_FM]
   const uint8_t* ext;    // [tile][nunits]
@@ -112,6 +113,7 @@ struct FoldArgs {
   int bn, nst;                  // positions per tile, ring depth
   int obufs;                    // output boxes per epilogue warp: 2 or 4
   int mtiles, ntiles, ktiles, nunits;
+  int uk, ux;                   // K-tiles from a unit's start to the next one's, and past that (plan_units)
   int out_tma;
   uint64_t timeout_ns;
 };
@@ -137,7 +139,7 @@ struct PrepFold {
   float* rs;
   uint8_t* ext;
   int wrow, ng, gshift;  // G = 1 << gshift
-  int Mg, Cg, cpad, mtiles, ktiles, nunits, nsub, fold_blocks;
+  int Mg, Cg, cpad, mtiles, ktiles, nunits, uk, ux, nsub, fold_blocks;
   int third;             // every unit carries the third part
   int quads;             // Cg % 4 == 0: 4 elements from a multiple of 4 lie in one tap and one group
   int padded;            // activations need the padded expansion
@@ -146,7 +148,7 @@ struct PrepFold {
   int64_t npix;          // pixels of the expanded activations
 };
 
-constexpr int PF_GPU = TF_UNIT * TF_KT / 4 + 2;  // groups a unit can touch (G >= 4), and one pad word
+constexpr int PF_GPU = TF_UNIT * TF_KT / 4 + 2;  // groups of a unit, at most 65, and a pad word
 
 __device__ __forceinline__ uint32_t h2u(float v) { return (uint32_t)__half_as_ushort(__float2half_rn(v)); }
 
@@ -258,13 +260,17 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
   const int tu = (int)blockIdx.x / f.nsub;
   const int tile = tu / f.nunits, u = tu - tile * f.nunits;
   const int gi = tile / f.mtiles, mt = tile - gi * f.mtiles;
-  const int kt0 = u * TF_UNIT;
-  const int kt1 = kt0 + TF_UNIT < f.ktiles ? kt0 + TF_UNIT : f.ktiles;
-  // the unit's real reduction indices are one range [k0, k1): padding follows a tap's channels
-  const int tap0 = kt0 * TF_KT / f.cpad, c0 = kt0 * TF_KT - tap0 * f.cpad;
-  const int tap1 = kt1 * TF_KT / f.cpad, c1 = kt1 * TF_KT - tap1 * f.cpad;
-  const int k0 = tap0 * f.Cg + (c0 < f.Cg ? c0 : f.Cg), k1 = tap1 * f.Cg + (c1 < f.Cg ? c1 : f.Cg);
-  const int g0 = k0 >> f.gshift, g1 = ((k1 - 1) >> f.gshift) + 1;  // k1 > k0: a K-tile holds real channels
+  const int kt0 = u * f.uk;
+  // the unit's groups [g0, g1): those that begin in its own uk K-tiles.  The last may run into the
+  // K-tiles after them (ux), whose other groups are left to the next unit.
+  auto real = [&](int kt) {  // real reduction elements ahead of K-tile kt
+    const int tap = kt * TF_KT / f.cpad;
+    return tap * f.Cg + (kt * TF_KT - tap * f.cpad);
+  };
+  const int ge = (1 << f.gshift) - 1;
+  const int g0 = (real(kt0) + ge) >> f.gshift;
+  const int g1 = kt0 + f.uk < f.ktiles ? (real(kt0 + f.uk) + ge) >> f.gshift : f.ng;
+  const int kt1 = kt0 + f.uk + f.ux < f.ktiles ? kt0 + f.uk + f.ux : f.ktiles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   bool small = f.third != 0;
   float v[TF_FM / 8][3];  // 8 filters per warp, every load in flight at once
@@ -308,8 +314,9 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
   // 16-byte chunks of the images: chunk c (8 elements) of the operand rows of filter fl
   for (int kt = kt0 + sub; kt < kt1; kt += f.nsub) {
     const int tap = kt * TF_KT / f.cpad, cb = kt * TF_KT - tap * f.cpad;
-    uint8_t* img = f.a_op + ((int64_t)tile * f.ktiles + kt) * TF_A;
-    uint8_t* imx = f.a_ext + ((int64_t)tile * f.ktiles + kt) * TF_A;
+    const int64_t slot = ((int64_t)tile * f.nunits + u) * (f.uk + f.ux) + (kt - kt0);
+    uint8_t* img = f.a_op + slot * TF_A;
+    uint8_t* imx = f.a_ext + slot * TF_A;
 #pragma unroll
     for (int it = 0; it < TF_FM * 8 / 256; ++it) {
       const int idx = (int)threadIdx.x + 256 * it;
@@ -330,9 +337,10 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
       if (f.quads) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          const uint32_t c4 = (cw >> (8 * q)) & 0xffu;
+          const int gr = ((k + 4 * q) >> f.gshift) - g0;
+          const uint32_t c4 = (uint32_t)gr < (uint32_t)(g1 - g0) ? (cw >> (8 * q)) & 0xffu : 0u;
           uint32_t hi = 0u, lo = 0u, third = 0u;
-          if (c4) split3(al[fl][((k + 4 * q) >> f.gshift) - g0], hi, lo, third);
+          if (c4) split3(al[fl][gr], hi, lo, third);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t c2 = (c4 >> (4 * h)) & 15u;
@@ -349,9 +357,10 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
           for (int h = 0; h < 2; ++h) {
             const int e = 2 * e2 + h;
             const uint32_t t = (cw >> (2 * e)) & 3u;  // 00 = 0, 01 = +1, 11 = -1
-            if (t) {
+            const int gr = ((k + e) >> f.gshift) - g0;
+            if (t && (uint32_t)gr < (uint32_t)(g1 - g0)) {
               uint32_t hi, lo, third;
-              split3(al[fl][((k + e) >> f.gshift) - g0], hi, lo, third);
+              split3(al[fl][gr], hi, lo, third);
               const uint32_t sgn = t == 3u ? 0x8000u : 0u;
               p0[e2] |= (hi ^ sgn) << (16 * h);
               p1[e2] |= (lo ^ sgn) << (16 * h);
@@ -452,13 +461,14 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
         w0 = wo * g.stride - g.pad;
       }
       int tr = 0, ts = 0, tc0 = 0;
-      for (int u = 0, kt0 = 0; u < a.nunits && ok; ++u, kt0 += TF_UNIT) {
-        const int nk = a.ktiles - kt0 < TF_UNIT ? a.ktiles - kt0 : TF_UNIT;
+      int ntr = 0, nts = 0, ntc = 0;  // where the next unit begins
+      for (int u = 0, kt0 = 0; u < a.nunits && ok; ++u, kt0 += a.uk) {
+        const int nk = a.ktiles - kt0 < a.uk + a.ux ? a.ktiles - kt0 : a.uk + a.ux;
         const int passes = 1 + next_ext;
         if (u + 1 < a.nunits) next_ext = __ldg(xp + u + 1);
-        const int utr = tr, uts = ts, utc = tc0;
+        const int utr = ntr, uts = nts, utc = ntc;
         for (int pass = 0; pass < passes && ok; ++pass) {
-          const uint8_t* asrc = (pass ? a.a_ext : a.a_op) + ((int64_t)gm * a.ktiles + kt0) * TF_A;
+          const uint8_t* asrc = (pass ? a.a_ext : a.a_op) + ((int64_t)gm * a.nunits + u) * (a.uk + a.ux) * TF_A;
           tr = utr;
           ts = uts;
           tc0 = utc;
@@ -490,6 +500,11 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
                 ++tr;
               }
             }
+            if (j == a.uk - 1) {
+              ntr = tr;
+              nts = ts;
+              ntc = tc0;
+            }
           }
         }
       }
@@ -516,8 +531,8 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
       fold_tile(a, t, gm, pt);
       const uint8_t* xp = a.ext + (int64_t)gm * a.nunits;
       int next_ext = __ldg(xp);  // the unit's mark, loaded one unit ahead
-      for (int u = 0, kt0 = 0; u < a.nunits && ok; ++u, kt0 += TF_UNIT) {
-        const int nk = a.ktiles - kt0 < TF_UNIT ? a.ktiles - kt0 : TF_UNIT;
+      for (int u = 0, kt0 = 0; u < a.nunits && ok; ++u, kt0 += a.uk) {
+        const int nk = a.ktiles - kt0 < a.uk + a.ux ? a.ktiles - kt0 : a.uk + a.ux;
         const int passes = 1 + next_ext;
         if (u + 1 < a.nunits) next_ext = __ldg(xp + u + 1);
         for (int pass = 0; pass < passes; ++pass, ++uc) {
@@ -724,10 +739,45 @@ int choose_bn(int64_t P, int wtiles, int ktiles, int sms) {
   return best;
 }
 
+// Units of a reduction: uk K-tiles each, and ux more where a unit's last group runs past them (a K-tile
+// starts inside a group where a tap's channels are no multiple of G: 3x3 over 72 channels at G = 32).  Every
+// group is summed in one unit: its halves in two would carry two roundings and two scales of its alpha,
+// as large as the halves themselves where these cancel.  Four K-tiles where that fits, else the number
+// up to eight that takes the fewest K-tiles in all; false where none fits.
+bool plan_units(const Geom& g, int kpt, int ktiles, int& uk, int& ux) {
+  int best = INT32_MAX;
+  for (int n = TF_UNIT; n <= TF_MAX_UNIT; ++n) {
+    if (n != TF_UNIT && n * TF_KT / g.G + 1 >= PF_GPU) break;
+    int x = 0, tiles = 0;
+    for (int kt = n; g.Cg % g.G != 0 && kt < ktiles; kt += n) {
+      int rem = (g.G - (kt / kpt * g.Cg + kt % kpt * TF_KT) % g.G) % g.G, t = 0;
+      for (; rem > 0 && kt + t < ktiles; ++t) {
+        const int c = g.Cg - (kt + t) % kpt * TF_KT;
+        rem -= c < TF_KT ? c : TF_KT;
+      }
+      if (t > x) x = t;
+    }
+    if (n + x > TF_MAX_UNIT) continue;
+    for (int kt = 0; kt < ktiles; kt += n) tiles += ktiles - kt < n + x ? ktiles - kt : n + x;
+    if (tiles < best) {
+      best = tiles;
+      uk = n;
+      ux = x;
+    }
+    if (x == 0) break;  // (a larger unit takes no fewer K-tiles)
+  }
+  return best < INT32_MAX;
+}
+
+int fold_ktiles_per_tap(const Geom& g) { return (g.Cg + TF_KT - 1) / TF_KT; }
+
 }  // namespace
 
 bool fold_supports(const Geom& g) {
   if (g.G < 4 || g.G > 64 || (g.G & (g.G - 1)) != 0) return false;
+  int uk, ux;
+  const int kpt = fold_ktiles_per_tap(g);
+  if (!plan_units(g, kpt, g.R * g.S * kpt, uk, ux)) return false;
   if (g.P >= (int64_t)1 << 31) return false;  // positions decoded in 32 bits
   if (tc::encode_tiled() == nullptr) return false;
   return tc::act_pointwise(g) || (tc::encode_im2col() != nullptr && tc::im2col_fits(g.R, g.S, g.stride, g.pad));
@@ -742,9 +792,10 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   a.out = out;
   a.err = err;
   a.g = g;
-  a.cpad = (g.Cg + TF_KT - 1) / TF_KT * TF_KT;
+  a.cpad = fold_ktiles_per_tap(g) * TF_KT;
   a.ktiles = g.R * g.S * (a.cpad / TF_KT);
-  a.nunits = (a.ktiles + TF_UNIT - 1) / TF_UNIT;
+  if (!plan_units(g, a.cpad / TF_KT, a.ktiles, a.uk, a.ux)) return FGQ_ERR_UNSUPPORTED;
+  a.nunits = (a.ktiles + a.uk - 1) / a.uk;
   a.mtiles = (g.Mg + TF_FM - 1) / TF_FM;
   const int wtiles = g.groups * a.mtiles;
   const int sms = num_sms();
@@ -767,7 +818,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   const bool pointwise = tc::act_pointwise(g);
   const int64_t npix = pointwise && g.stride > 1 ? g.P : (int64_t)g.B * g.H * g.W;
   const int64_t ca = (int64_t)g.groups * a.cpad;
-  const size_t a_bytes = (size_t)wtiles * a.ktiles * TF_A;
+  const size_t a_bytes = (size_t)wtiles * a.nunits * (a.uk + a.ux) * TF_A;
   const size_t rs_bytes = ((size_t)wtiles * a.nunits * TF_FM * 4 + 255) / 256 * 256;
   const size_t ext_bytes = ((size_t)wtiles * a.nunits + 255) / 256 * 256;
   const size_t x_bytes = (size_t)npix * ca * 2;
@@ -793,6 +844,8 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.mtiles = a.mtiles;
   f.ktiles = a.ktiles;
   f.nunits = a.nunits;
+  f.uk = a.uk;
+  f.ux = a.ux;
   f.nsub = wtiles * a.nunits >= 2 * sms ? 1 : TF_UNIT;
   f.third = g.G > 4 && g.ng < FOLD_FEW_GROUPS ? 1 : 0;
   f.quads = g.Cg % 4 == 0 ? 1 : 0;

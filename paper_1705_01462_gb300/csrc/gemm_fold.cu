@@ -6,22 +6,23 @@
 // t[m][k], if it can be summed without losing what the 32-bit group accumulators of Section 4
 // keep.  Here it can, because the folded weights are integers on a common grid: the reduction
 // is cut into units of about 256 elements and whole groups (plan_units), and in each unit row m is
-// scaled by a power of two 2^e that puts its largest alpha into (2^10, 2^11]; with v = alpha 2^e,
-//     hi = rint(v),   lo = fp16((v - hi) 2^12),
-// both exact in fp16 (hi an integer of magnitude <= 2048).  Products hi t q are integers below
-// 2^19, so a unit's sum over 256 of them is the exact integer as long as it stays below 2^24 --
-// in any order, whatever cancels -- and beyond that each of the unit's 16 accumulations rounds
-// a prefix sum of whole groups by at most 2^-23 of itself.  What the pair (hi, lo) leaves out
-// is at most 2^-13 of v's unit: 2^-24 of the unit's largest alpha (the fp32 alphas themselves
-// carry 2^-24).  Against |y| bounded by S = s_x sum_g |alpha_g s_g| that is
-//     16 2^-23 (accumulator) + 2^-13 / min v (alphas) + n_units 2^-24 (fp32 adds of the units)
-// of S; with min v >= 16 and at most 16384 products it is below 1e-5.  A unit in which some
-// filter of the tile holds a non-zero alpha with v < 16 (more than 64 times below the row's
-// largest) gets a third part, fp16 of what (hi, lo) leave out times 2^24, contracted in a pass
-// of its own over the unit: then every alpha is carried to 22 bits or more.  The preparation
+// scaled by a power of two 2^e that puts its largest alpha into [2^10, 2^11) ([2^9, 2^10) at G = 64);
+// with v = alpha 2^e and d = 12 (11 at G = 64),
+//     hi = rint(v),   lo = rint((v - hi) 2^d),
+// integers of magnitude at most 2^(d - 1), exact in fp16.  Products with 8-bit codes are integers,
+// and so are their sums, exact in the fp32 accumulator below 2^24, in any order, whatever
+// cancels.  What an accumulator holds of whole groups is bounded by their own |alpha s|, what it
+// holds of a group half summed by 2^23 (32 products of 255 with 2^10 at G = 64, 16 with 2^11 at
+// G = 32), however much of that the other half takes back: a prefix that passes 2^24 has more than
+// 2^23 from S = s_x sum_g |alpha_g s_g| in it, and rounding it costs at most 2^-22 of S in each of
+// a unit's 16 to 32 accumulations.  What the pair (hi, lo) leaves out of an alpha is at most
+// 2^-(d + 1) of v's unit: 2^-13, or 2^-24 of the unit's largest alpha (the fp32 alphas themselves
+// carry 2^-24).  A unit in which some filter of the tile holds a non-zero alpha with v < 16 (more than
+// 64 times below the row's largest) gets a third part, rint of what (hi, lo) leave out times 2^(2 d),
+// contracted in a pass of its own over the unit.  The preparation
 // marks such units (about 1 in 300 for Gaussian weights at G = 4, rarer for larger G), and at G >= 8
 // all units of layers with few groups (FOLD_FEW_GROUPS), whose few fp32 adds err less than two
-// parts of the alphas would.
+// parts of the alphas would, and all at G = 64, where two parts have 22 bits.
 //
 // hi and lo are two rows of the same MMA operand: a tile is 64 filters x up to 256 positions,
 // 128 operand rows (rows 32 q + i and 32 q + 16 + i: hi and lo of filter 16 q + i), so that one
@@ -72,6 +73,8 @@ using tc::make_map_im2col;
 constexpr int TF_ROWS = 128;      // MMA M
 constexpr int TF_FM = 64;         // filters per tile (two operand rows each)
 constexpr int TF_KT = 64;         // reduction elements per K-tile: 4 MMAs
+constexpr int TF_DIGIT = 12;      // bits of an alpha's part: integers up to 2048.  11 at G = 64, so that half a
+                                  // group, 32 products of 255 with the largest alpha, is 2^23 there too
 constexpr int TF_UNIT = 4;        // K-tiles per unit (one TMEM accumulation) where its groups allow it,
 constexpr int TF_MAX_UNIT = 8;    // and at most (plan_units)
 constexpr int TF_MAX_BN = 256;    // positions per tile (MMA N), a multiple of 64
@@ -112,6 +115,7 @@ struct FoldArgs {
   int cpad;                     // channels per conv group in the padded activations
   int bn, nst;                  // positions per tile, ring depth
   int obufs;                    // output boxes per epilogue warp: 2 or 4
+  float lo_scale, ext_scale;    // 2^-dbits, 2^-(2 dbits)
   int mtiles, ntiles, ktiles, nunits;
   int uk, ux;                   // K-tiles from a unit's start to the next one's, and past that (plan_units)
   int out_tma;
@@ -139,6 +143,7 @@ struct PrepFold {
   float* rs;
   uint8_t* ext;
   int wrow, ng, gshift;  // G = 1 << gshift
+  int dbits;             // bits of a part
   int Mg, Cg, cpad, mtiles, ktiles, nunits, uk, ux, nsub, fold_blocks;
   int third;             // every unit carries the third part
   int quads;             // Cg % 4 == 0: 4 elements from a multiple of 4 lie in one tap and one group
@@ -226,14 +231,15 @@ __device__ __forceinline__ void expand_padded(const PrepFold& f, const prep::Act
   }
 }
 
-// hi and lo (and the third part) of one scaled alpha, as fp16 bits.
-__device__ __forceinline__ void split3(float v, uint32_t& hi, uint32_t& lo, uint32_t& third) {
+// hi and lo (and the third part) of one scaled alpha, as fp16 bits: digits of log2(digit) bits, each an
+// integer of magnitude at most digit / 2 <= 2048 (exact in fp16).
+__device__ __forceinline__ void split3(float v, float digit, uint32_t& hi, uint32_t& lo, uint32_t& third) {
   const float h = rintf(v);
-  const float r1 = (v - h) * 4096.0f;
-  const __half l = __float2half_rn(r1);
+  const float r1 = (v - h) * digit;
+  const float l = rintf(r1);
   hi = h2u(h);
-  lo = (uint32_t)__half_as_ushort(l);
-  third = h2u((r1 - __half2float(l)) * 4096.0f);
+  lo = h2u(l);
+  third = h2u(rintf((r1 - l) * digit));
 }
 
 // The fp16 pair (x, x) with the signs and zeros of two codes (4 bits: 00 = 0, 01 = +1, 11 = -1).
@@ -272,6 +278,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
   const int g1 = kt0 + f.uk < f.ktiles ? (real(kt0 + f.uk) + ge) >> f.gshift : f.ng;
   const int kt1 = kt0 + f.uk + f.ux < f.ktiles ? kt0 + f.uk + f.ux : f.ktiles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float digit = (float)(1 << f.dbits);
   bool small = f.third != 0;
   float v[TF_FM / 8][3];  // 8 filters per warp, every load in flight at once
 #pragma unroll
@@ -298,8 +305,8 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
     }
-    // 2^e puts the largest alpha into [2^10, 2^11); e is kept where 2^e and 2^-e are normal
-    int e = mx > 0.0f ? 10 - ilogbf(mx) : 0;
+    // 2^e puts the largest alpha into [digit / 4, digit / 2); e is kept where 2^e and 2^-e are normal
+    int e = mx > 0.0f ? f.dbits - 2 - ilogbf(mx) : 0;
     e = e < -120 ? -120 : (e > 120 ? 120 : e);
     const float mul = pow2f(e);
     if (mx > 0.0f && mn * mul < 16.0f) small = true;
@@ -340,7 +347,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
           const int gr = ((k + 4 * q) >> f.gshift) - g0;
           const uint32_t c4 = (uint32_t)gr < (uint32_t)(g1 - g0) ? (cw >> (8 * q)) & 0xffu : 0u;
           uint32_t hi = 0u, lo = 0u, third = 0u;
-          if (c4) split3(al[fl][gr], hi, lo, third);
+          if (c4) split3(al[fl][gr], digit, hi, lo, third);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t c2 = (c4 >> (4 * h)) & 15u;
@@ -360,7 +367,7 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
             const int gr = ((k + e) >> f.gshift) - g0;
             if (t && (uint32_t)gr < (uint32_t)(g1 - g0)) {
               uint32_t hi, lo, third;
-              split3(al[fl][gr], hi, lo, third);
+              split3(al[fl][gr], digit, hi, lo, third);
               const uint32_t sgn = t == 3u ? 0x8000u : 0u;
               p0[e2] |= (hi ^ sgn) << (16 * h);
               p1[e2] |= (lo ^ sgn) << (16 * h);
@@ -587,7 +594,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
     const int fl = 16 * quarter + (lane & 15);  // filter of the tile
     const int hcols = a.bn / 2;                 // positions of this warp (a multiple of 32)
     const uint32_t tbase = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(hcols * half);
-    const float sx = __ldg(a.act_scale);
+    const float sx = __ldg(a.act_scale), lo_scale = a.lo_scale;
     int b = 0, obuf = 0;
     uint32_t fph = 0;
     bool ok = true;
@@ -614,7 +621,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
         }
         for (int pass = 0; pass < passes; ++pass) {
           if (!ok) continue;  // after a failed wait: run out the tile, then leave with the others
-          const float r = pass ? r0 * 0x1p-24f : r0;  // the third part (in hi's rows) carries 2^24
+          const float r = pass ? r0 * a.ext_scale : r0;  // the third part (in hi's rows)
           if (!mbar_wait_warp(&acc_full[b], fph, tmo, abort_flag)) {
             ok = false;
             continue;
@@ -632,7 +639,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
 #pragma unroll
               for (int i = 0; i < 16; ++i)
                 acc[16 * j + i] =
-                    fmaf(r, fmaf(0x1p-12f, __uint_as_float(dl[i]), __uint_as_float(dh[i])), acc[16 * j + i]);
+                    fmaf(r, fmaf(lo_scale, __uint_as_float(dl[i]), __uint_as_float(dh[i])), acc[16 * j + i]);
             }
           }
           tc_fence_before();
@@ -838,6 +845,9 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.wrow = g.wrow;
   f.ng = g.ng;
   f.gshift = 31 - __builtin_clz((unsigned)g.G);
+  f.dbits = g.G > 32 ? TF_DIGIT - 1 : TF_DIGIT;
+  a.lo_scale = 1.0f / (float)(1 << f.dbits);
+  a.ext_scale = a.lo_scale * a.lo_scale;
   f.Mg = g.Mg;
   f.Cg = g.Cg;
   f.cpad = a.cpad;
@@ -847,7 +857,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.uk = a.uk;
   f.ux = a.ux;
   f.nsub = wtiles * a.nunits >= 2 * sms ? 1 : TF_UNIT;
-  f.third = g.G > 4 && g.ng < FOLD_FEW_GROUPS ? 1 : 0;
+  f.third = g.G > 32 || (g.G > 4 && g.ng < FOLD_FEW_GROUPS) ? 1 : 0;
   f.quads = g.Cg % 4 == 0 ? 1 : 0;
   f.padded = (a.cpad != g.Cg || g.C % 16 != 0) ? 1 : 0;
   f.fast8 = f.padded && g.Cg % 8 == 0 && g.C % 8 == 0 && (g.act_type == FGQ_U8 || g.act_type == FGQ_S8) ? 1 : 0;

@@ -59,3 +59,31 @@ def test_fold_groups_cut_by_taps(C, G, R):
     assert fgq.fgq_last_path() == fgq.PATH_TC
     check_within(got, y, ym, f"groups cut by taps C={C} G={G}")
     assert np.all(got[ym == 0] == 0)
+
+
+@pytest.mark.parametrize("G", [8, 16, 32, 64])
+def test_fold_sums_inside_groups(G):
+    """What an accumulator holds between the two halves of a group that cancels: at G = 64 32 products of
+    255 with the largest alpha, 2^24 on the grid of 2^11.  A filter's output is one group's sum of 37
+    with alphas whose grid value is odd, so that a unit lost there is 1.3e-5 of it; filters of
+    cancelling groups alone, with alphas of many magnitudes, give exactly zero."""
+    rng = np.random.default_rng(G)
+    P, K, M = 140, 1184, 96
+    ng = -(-K // G)
+    al = np.full((M, ng), 1.999, np.float32)
+    al[M // 2:] = rng.uniform(0.02, 2.0, (M // 2, ng))
+    tg = np.tile(np.concatenate([np.ones(G // 2), -np.ones(G // 2)]).astype(np.int8), (M, ng, 1))
+    tg[:, ::4] = 0  # every fourth group holds one code in one filter, and nothing in the others
+    if K % G:
+        tg[:, -1] = 0
+    q = np.full((P, K), 255, np.int32)
+    q[1::2] = rng.integers(200, 256, (P // 2, 1))
+    q[:, ::4 * G] = 37
+    for m in range(0, M, 2):
+        tg[m, 4 * (m // 2 % ((K // G + 3) // 4)), 0] = 1
+    t = tg.reshape(M, -1)
+    y, ym = O.gemm(q, np.float32(1.0), t, al, G)
+    got = _conv(q.reshape(P, 1, 1, K), "u8", t, al, G, 1, 1).reshape(P, M)
+    assert fgq.fgq_last_path() == fgq.PATH_TC
+    check_within(got, y, ym, f"sums inside groups G={G}")
+    assert np.all(got[ym == 0] == 0)

@@ -95,17 +95,13 @@ bool tc4_supports(const Geom& g);
 fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes, int32_t* sums, unsigned int* err,
                            cudaStream_t s);
 
-// Tensor-core contraction for G in {4, 8, 16, 32}: the alphas folded into integer weights on a
-// common grid per 256 reduction elements, in two fp16 parts.  Any channel count, 8- or 4-bit
-// activations.
-// With fewer groups per filter than this, fp32 adds of the exact group sums (dp4a) err less than two
-// fp16 parts of the alphas: the folded kernel then carries a third part (G = 8 to 32) or is not used
-// (G = 64; nor where its units, padded to whole K-tiles, are more than 2 / 5 of the groups).  Error against 64 bits, root mean square, of dp4a / two parts / three parts: G = 64,
-// 6 groups 4.8e-8 / 6.4e-8 / 5.0e-8, 11 6.5e-8 / 7.6e-8 / 6.1e-8, 14 6.9e-8 / 7.7e-8 / 5.9e-8, 19 7.9e-8 /
-// 7.1e-8, 29 9.6e-8 / 7.6e-8; G = 128 (not taken), 18 groups in 12 units
-// 7.5e-8 / 8.6e-8; G = 32,
-// dp4a / three parts, 8 groups 5.3e-8 / 3.4e-8, 16 7.3e-8 / 4.4e-8.  The third part costs 3x3 64 -> 64 on 56 x 56, batch 64, G = 32 41 us
-// (dp4a 155), 1x1 512 -> 128 on 28 x 28 42 (85).
+// Tensor-core contraction for G in {4, 8, 16, 32, 64}: the alphas folded into the weights on a common
+// grid per about 256 reduction elements, in one or two pairs of fp16 parts.  Any channel count, 8- or
+// 4-bit activations.  At G = 64 the automatic choice takes it from FOLD_FEW_GROUPS groups per filter on, and
+// only where its units of four K-tiles (each two fp32 adds) are no more than 2 / 5 of the groups: fp32 adds
+// of fewer exact group sums (dp4a) err about as little.  Error against 64 bits, root mean square, of
+// dp4a / this kernel at G = 64: 19 groups 8.4e-8 / 8.1e-8, 21 8.8e-8 / 6.5e-8, 24 9.0e-8 / 8.1e-8,
+// 29 9.6e-8 / 7.3e-8, 50 12.5e-8 / 9.1e-8.
 constexpr int FOLD_FEW_GROUPS = 18;
 bool fold_supports(const Geom& g);
 fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,

@@ -8,31 +8,49 @@
 // is cut into units of about 256 elements and whole groups (plan_units), and in each unit row m is
 // scaled by a power of two 2^e that puts its largest alpha into [2^10, 2^11) ([2^9, 2^10) at G = 64);
 // with v = alpha 2^e and d = 12 (11 at G = 64),
-//     hi = rint(v),   lo = rint((v - hi) 2^d),
-// integers of magnitude at most 2^(d - 1), exact in fp16.  Products with 8-bit codes are integers,
-// and so are their sums, exact in the fp32 accumulator below 2^24, in any order, whatever
-// cancels.  What an accumulator holds of whole groups is bounded by their own |alpha s|, what it
-// holds of a group half summed by 2^23 (32 products of 255 with 2^10 at G = 64, 16 with 2^11 at
-// G = 32), however much of that the other half takes back: a prefix that passes 2^24 has more than
-// 2^23 from S = s_x sum_g |alpha_g s_g| in it, and rounding it costs at most 2^-22 of S in each of
-// a unit's 16 to 32 accumulations.  What the pair (hi, lo) leaves out of an alpha is at most
-// 2^-(d + 1) of v's unit: 2^-13, or 2^-24 of the unit's largest alpha (the fp32 alphas themselves
-// carry 2^-24).  A unit in which some filter of the tile holds a non-zero alpha with v < 16 (more than
-// 64 times below the row's largest) gets a third part, rint of what (hi, lo) leave out times 2^(2 d),
-// contracted in a pass of its own over the unit.  The preparation
-// marks such units (about 1 in 300 for Gaussian weights at G = 4, rarer for larger G), and at G >= 8
-// all units of layers with few groups (FOLD_FEW_GROUPS), whose few fp32 adds err less than two
-// parts of the alphas would, and all at G = 64, where two parts have 22 bits.
+//     hi = round(v),   lo = round((v - hi) 2^d),
+// fp16 numbers of magnitude at most 2^(d - 1) on a grid of 2^-f (and of their own ulp).
+//
+// f = 0, integers, where a group may reach over several MMA steps (G >= 32, or channels that are no
+// multiple of G).  Products with 8-bit codes are integers, and so are their sums, exact in the fp32
+// accumulator below 2^24, in any order, whatever cancels.  What an accumulator holds of whole
+// groups is bounded by their own |alpha s|, what it holds of a group half summed by 2^23 (32
+// products of 255 with 2^10 at G = 64, 16 with 2^11 at G = 32), however much of that the other half
+// takes back: a prefix that passes 2^24 has more than 2^23 from S = s_x sum_g |alpha_g s_g| in it, and
+// rounding it costs at most 2^-22 of S in each of a unit's 16 to 32 accumulations.
+//
+// f = 6 where every group lies inside one MMA step of 16 elements: the accumulator then holds whole
+// groups only, and a step adds its 16 products and the accumulator without loss between 2^19, the
+// largest, and 2^-8 (found exact on this chip, and tested down to 2^-6 of products next to
+// cancelling ones of 2^19; a narrower sum would lose what a large group leaves behind).  Alphas down to
+// 2^-7 of the largest then keep 22 bits in one pair.
+//
+// What the pair (hi, lo) leaves out of an alpha at f = 0 is at most 2^-(d + 1) of v's unit: 2^-13, or
+// 2^-24 of the unit's largest alpha, but more of a smaller one.  A unit in which some alpha of the
+// tile's 64 filters loses more than pair_tolerance of itself gets a second pair, the next two digits of
+// the same rule, contracted in a pass of its own over the unit: 47 bits of the largest alpha in all (43
+// at G = 64), every bit of alphas down to 2^-23 (2^-19) of it and 18 bits down to 2^-29 (2^-25).
+// The tolerance keeps the output's error no larger than that of fp32 alphas on exact group sums,
+// also where a row's large alphas meet inactive channels.  Gaussian weights: no unit at f = 6 where a
+// filter has 20 groups more than three per unit, else all; at G = 32 and 64 nearly all.
+// (Integers in one pair, and a third part only from alphas 64 times below the largest on, erred by
+// 2.6e-6 where dp4a errs by 4.4e-7: one large alpha in 256 elements with zero activations, the others
+// 45 times smaller.  Integers for all G, in two pairs wherever the tolerance asks, at G = 4 everywhere,
+// took 48 us for the first call below and 366 for the fourth.)
+// Against S the error is below 16 2^-22 (accumulations of four K-tiles) + 2^-20 (alphas of one pair) +
+// n_units 2^-24 for each pair (fp32 adds): 1e-5 up to 88 units of one pair or 52 of two, if every rounding
+// goes the same way; measured it is 1e-7.
 //
 // hi and lo are two rows of the same MMA operand: a tile is 64 filters x up to 256 positions,
 // 128 operand rows (rows 32 q + i and 32 q + 16 + i: hi and lo of filter 16 q + i), so that one
 // epilogue warp reads both parts of its 16 filters (adding them across lanes by shuffles cost
 // more than the rest of the tile end).  The MMA work is
-// twice the dense contraction's.  (A block-diagonal operand with a row per group slot, used at
-// G = 4 before, did eight times the dense work, drained TMEM every K-tile and wrote 16 bytes of
-// operand per weight.  A call before and now, us: 3x3 128 -> 128 on 28 x 28, batch 64, G = 4: 82 ->
-// 34; 3x3 256 -> 256 on 14 x 14, batch 64, G = 8 (dp4a before): 236 -> 34; 5x5 with 2 x 48 channels on
-// 27 x 27, batch 256, G = 4 (dp4a before): 2661 -> 208; GEMM 4096 x 9216, P = 256, G = 4: 555 -> 87.)
+// twice the dense contraction's for each pair.  (A block-diagonal operand with a row per group slot,
+// used at G = 4 before, did eight times the dense work, drained TMEM every K-tile and wrote 16 bytes of
+// operand per weight.  A call before and now, us: 3x3 128 -> 128 on 28 x 28, batch 64, G = 4: 82 and
+// 33; 3x3 256 -> 256 on 14 x 14, batch 64, G = 8 (dp4a before): 236 and 32, and with two pairs, G = 32,
+// 179 and 54; 5x5 with 2 x 48 channels on 27 x 27, batch 256, G = 4 (dp4a before): 2661 and 207, with two
+// pairs, G = 64, 1742 and 366; GEMM 4096 x 9216, P = 256, G = 4: 555 and 89.)
 // Bound: the tensor pipe for long reductions (512 clk per 64 x 256 x 64 K-tile pair), the stores
 // of the tile end for short ones.
 //
@@ -58,6 +76,7 @@
 // TMEM is freed.
 #include <cuda_fp16.h>
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -75,6 +94,7 @@ constexpr int TF_FM = 64;         // filters per tile (two operand rows each)
 constexpr int TF_KT = 64;         // reduction elements per K-tile: 4 MMAs
 constexpr int TF_DIGIT = 12;      // bits of an alpha's part: integers up to 2048.  11 at G = 64, so that half a
                                   // group, 32 products of 255 with the largest alpha, is 2^23 there too
+constexpr int TF_FRAC = 6;        // fractional bits of a part where groups lie inside MMA steps
 constexpr int TF_UNIT = 4;        // K-tiles per unit (one TMEM accumulation) where its groups allow it,
 constexpr int TF_MAX_UNIT = 8;    // and at most (plan_units)
 constexpr int TF_MAX_BN = 256;    // positions per tile (MMA N), a multiple of 64
@@ -105,7 +125,7 @@ struct FoldArgs {
   CUtensorMap act_map;   // fp16 activations: 2D [positions][Ca] or im2col, box 64 channels x bn positions
   CUtensorMap out_map;   // out_tma: outputs [P][M] (fp32 or codes), box {16 filters, 32 positions}
   const uint8_t* a_op;   // weight K-tile images [tile][nunits][uk + ux] of TF_A bytes
-  const uint8_t* a_ext;  // the third parts, same layout (written where ext is set)
+  const uint8_t* a_ext;  // the second pairs, same layout (written where ext is set)
   const float* rs;       // 2^-e [tile][nunits][TF_FM]
   const uint8_t* ext;    // [tile][nunits]
   const float* act_scale;
@@ -143,9 +163,9 @@ struct PrepFold {
   float* rs;
   uint8_t* ext;
   int wrow, ng, gshift;  // G = 1 << gshift
-  int dbits;             // bits of a part
+  int dbits, fbits;      // bits of a part; fractional bits
   int Mg, Cg, cpad, mtiles, ktiles, nunits, uk, ux, nsub, fold_blocks;
-  int third;             // every unit carries the third part
+  float tol;             // share of an alpha that one pair of parts may leave out
   int quads;             // Cg % 4 == 0: 4 elements from a multiple of 4 lie in one tap and one group
   int padded;            // activations need the padded expansion
   int fast8;             // ... of 8-bit codes in aligned runs of 8 (Cg and C multiples of 8)
@@ -231,15 +251,19 @@ __device__ __forceinline__ void expand_padded(const PrepFold& f, const prep::Act
   }
 }
 
-// hi and lo (and the third part) of one scaled alpha, as fp16 bits: digits of log2(digit) bits, each an
-// integer of magnitude at most digit / 2 <= 2048 (exact in fp16).
-__device__ __forceinline__ void split3(float v, float digit, uint32_t& hi, uint32_t& lo, uint32_t& third) {
-  const float h = rintf(v);
-  const float r1 = (v - h) * digit;
-  const float l = rintf(r1);
-  hi = h2u(h);
-  lo = h2u(l);
-  third = h2u(rintf((r1 - l) * digit));
+// The fp16 number next to v on a grid of 1 / frac, which is finer than fp16 itself from 1024 / frac on.
+__device__ __forceinline__ __half grid_half(float v, float frac, float unfrac) {
+  return __float2half_rn(fabsf(v) < 1024.0f * unfrac ? rintf(v * frac) * unfrac : v);
+}
+
+// The two parts of a scaled alpha, fp16 bits of hi and (above) lo; v becomes what they leave, times
+// digit^2: the next pair's v.
+__device__ __forceinline__ uint32_t split2(float& v, float digit, float frac, float unfrac) {
+  const __half h = grid_half(v, frac, unfrac);
+  const float r1 = (v - __half2float(h)) * digit;
+  const __half l = grid_half(r1, frac, unfrac);
+  v = (r1 - __half2float(l)) * digit;
+  return (uint32_t)__half_as_ushort(h) | (uint32_t)__half_as_ushort(l) << 16;
 }
 
 // The fp16 pair (x, x) with the signs and zeros of two codes (4 bits: 00 = 0, 01 = +1, 11 = -1).
@@ -249,9 +273,10 @@ __device__ __forceinline__ uint32_t code_pair(uint32_t c, uint32_t x) {
   return ((x * 0x10001u) ^ sg) & nz;
 }
 
-__global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ PrepFold f,
+// Four blocks per SM: without that bound 74 registers and three, GEMM 4096 x 9216 51 us instead of 46.
+__global__ void __launch_bounds__(256, 4) prep_fold_kernel(const __grid_constant__ PrepFold f,
                                                         const __grid_constant__ prep::ActSrc src, uint4* __restrict__ x16) {
-  __shared__ float al[TF_FM][PF_GPU + 1];  // the unit's alphas, scaled: v = alpha 2^e
+  __shared__ uint32_t al[TF_FM][PF_GPU + 1];  // a pair of parts of each of the unit's alphas (split2)
   pdl_wait();
   pdl_trigger();
   if ((int)blockIdx.x >= f.fold_blocks) {
@@ -279,7 +304,9 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
   const int kt1 = kt0 + f.uk + f.ux < f.ktiles ? kt0 + f.uk + f.ux : f.ktiles;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float digit = (float)(1 << f.dbits);
-  bool small = f.third != 0;
+  const float frac = (float)(1 << f.fbits), unfrac = 1.0f / frac;
+  const float tol = f.tol * digit * digit;
+  bool wide = false;  // some alpha needs the second pair
   float v[TF_FM / 8][3];  // 8 filters per warp, every load in flight at once
 #pragma unroll
   for (int i = 0; i < TF_FM / 8; ++i) {
@@ -294,98 +321,96 @@ __global__ void __launch_bounds__(256) prep_fold_kernel(const __grid_constant__ 
 #pragma unroll
   for (int i = 0; i < TF_FM / 8; ++i) {
     const int fl = (TF_FM / 8) * warp + i;
-    float mx = 0.0f, mn = __int_as_float(0x7f800000);
+    float mx = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      mx = fmaxf(mx, fabsf(v[i][j]));
-      if (v[i][j] != 0.0f) mn = fminf(mn, fabsf(v[i][j]));
-    }
+    for (int j = 0; j < 3; ++j) mx = fmaxf(mx, fabsf(v[i][j]));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     // 2^e puts the largest alpha into [digit / 4, digit / 2); e is kept where 2^e and 2^-e are normal
     int e = mx > 0.0f ? f.dbits - 2 - ilogbf(mx) : 0;
     e = e < -120 ? -120 : (e > 120 ? 120 : e);
     const float mul = pow2f(e);
-    if (mx > 0.0f && mn * mul < 16.0f) small = true;
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      if (lane + 32 * j < PF_GPU) al[fl][lane + 32 * j] = v[i][j] * mul;  // exact: a power-of-two scaling
+    for (int j = 0; j < 3; ++j) {
+      const float x = v[i][j] * mul;  // exact: a power of two
+      v[i][j] = x;
+      const uint32_t parts = split2(v[i][j], digit, frac, unfrac);  // leaves the rest in v
+      if (fabsf(v[i][j]) > tol * fabsf(x)) wide = true;
+      if (lane + 32 * j < PF_GPU) al[fl][lane + 32 * j] = parts;
+    }
     if (sub == 0 && lane == 0) f.rs[((int64_t)tile * f.nunits + u) * TF_FM + fl] = pow2f(-e);
   }
-  const bool ext = __syncthreads_or(small);
+  const bool ext = __syncthreads_or(wide);
   if (sub == 0 && threadIdx.x == 0) f.ext[(int64_t)tile * f.nunits + u] = ext ? 1 : 0;
 
-  // 16-byte chunks of the images: chunk c (8 elements) of the operand rows of filter fl
-  for (int kt = kt0 + sub; kt < kt1; kt += f.nsub) {
-    const int tap = kt * TF_KT / f.cpad, cb = kt * TF_KT - tap * f.cpad;
-    const int64_t slot = ((int64_t)tile * f.nunits + u) * (f.uk + f.ux) + (kt - kt0);
-    uint8_t* img = f.a_op + slot * TF_A;
-    uint8_t* imx = f.a_ext + slot * TF_A;
+  for (int pair = 0;; ++pair) {
+    // 16-byte chunks of the images: chunk c (8 elements) of the operand rows of filter fl
+    for (int kt = kt0 + sub; kt < kt1; kt += f.nsub) {
+      const int tap = kt * TF_KT / f.cpad, cb = kt * TF_KT - tap * f.cpad;
+      uint8_t* img = (pair ? f.a_ext : f.a_op) + (((int64_t)tile * f.nunits + u) * (f.uk + f.ux) + (kt - kt0)) * TF_A;
 #pragma unroll
-    for (int it = 0; it < TF_FM * 8 / 256; ++it) {
-      const int idx = (int)threadIdx.x + 256 * it;
-      const int fl = idx >> 3, c = idx & 7;
-      const int local = mt * TF_FM + fl;
-      const int ch = cb + 8 * c;  // channel of the chunk's first element
-      const int nv = local < f.Mg ? f.Cg - ch : 0;  // real elements from here on
-      const int k = tap * f.Cg + ch;
-      uint32_t cw = 0u;
-      if (nv > 0) {
-        const uint32_t* cr = f.codes + ((int64_t)gi * f.Mg + local) * f.wrow + (k >> 4);
-        const uint32_t lo = __ldg(cr);
-        const uint32_t hi = (k & 15) > 8 && (k >> 4) + 1 < f.wrow ? __ldg(cr + 1) : 0u;
-        cw = __funnelshift_r(lo, hi, 2 * (k & 15));
-        cw &= nv < 8 ? (1u << (2 * nv)) - 1u : 0xffffu;
-      }
-      uint32_t p0[4], p1[4], p2[4];
-      if (f.quads) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int gr = ((k + 4 * q) >> f.gshift) - g0;
-          const uint32_t c4 = (uint32_t)gr < (uint32_t)(g1 - g0) ? (cw >> (8 * q)) & 0xffu : 0u;
-          uint32_t hi = 0u, lo = 0u, third = 0u;
-          if (c4) split3(al[fl][gr], digit, hi, lo, third);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t c2 = (c4 >> (4 * h)) & 15u;
-            p0[2 * q + h] = code_pair(c2, hi);
-            p1[2 * q + h] = code_pair(c2, lo);
-            p2[2 * q + h] = code_pair(c2, third);
-          }
+      for (int it = 0; it < TF_FM * 8 / 256; ++it) {
+        const int idx = (int)threadIdx.x + 256 * it;
+        const int fl = idx >> 3, c = idx & 7;
+        const int local = mt * TF_FM + fl;
+        const int ch = cb + 8 * c;  // channel of the chunk's first element
+        const int nv = local < f.Mg ? f.Cg - ch : 0;  // real elements from here on
+        const int k = tap * f.Cg + ch;
+        uint32_t cw = 0u;
+        if (nv > 0) {
+          const uint32_t* cr = f.codes + ((int64_t)gi * f.Mg + local) * f.wrow + (k >> 4);
+          const uint32_t lo = __ldg(cr);
+          const uint32_t hi = (k & 15) > 8 && (k >> 4) + 1 < f.wrow ? __ldg(cr + 1) : 0u;
+          cw = __funnelshift_r(lo, hi, 2 * (k & 15));
+          cw &= nv < 8 ? (1u << (2 * nv)) - 1u : 0xffffu;
         }
-      } else {
+        uint32_t p0[4], p1[4];
+        if (f.quads) {
 #pragma unroll
-        for (int e2 = 0; e2 < 4; ++e2) {
-          p0[e2] = p1[e2] = p2[e2] = 0u;
+          for (int q = 0; q < 2; ++q) {
+            const int gr = ((k + 4 * q) >> f.gshift) - g0;
+            const uint32_t c4 = (uint32_t)gr < (uint32_t)(g1 - g0) ? (cw >> (8 * q)) & 0xffu : 0u;
+            const uint32_t x = c4 ? al[fl][gr] : 0u;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int e = 2 * e2 + h;
-            const uint32_t t = (cw >> (2 * e)) & 3u;  // 00 = 0, 01 = +1, 11 = -1
-            const int gr = ((k + e) >> f.gshift) - g0;
-            if (t && (uint32_t)gr < (uint32_t)(g1 - g0)) {
-              uint32_t hi, lo, third;
-              split3(al[fl][gr], digit, hi, lo, third);
-              const uint32_t sgn = t == 3u ? 0x8000u : 0u;
-              p0[e2] |= (hi ^ sgn) << (16 * h);
-              p1[e2] |= (lo ^ sgn) << (16 * h);
-              p2[e2] |= (third ^ sgn) << (16 * h);
+            for (int h = 0; h < 2; ++h) {
+              const uint32_t c2 = (c4 >> (4 * h)) & 15u;
+              p0[2 * q + h] = code_pair(c2, x & 0xffffu);
+              p1[2 * q + h] = code_pair(c2, x >> 16);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int e2 = 0; e2 < 4; ++e2) {
+            p0[e2] = p1[e2] = 0u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int e = 2 * e2 + h;
+              const uint32_t t = (cw >> (2 * e)) & 3u;  // 00 = 0, 01 = +1, 11 = -1
+              const int gr = ((k + e) >> f.gshift) - g0;
+              if (t && (uint32_t)gr < (uint32_t)(g1 - g0)) {
+                const uint32_t x = al[fl][gr] ^ (t == 3u ? 0x80008000u : 0u);
+                p0[e2] |= (x & 0xffffu) << (16 * h);
+                p1[e2] |= (x >> 16) << (16 * h);
+              }
             }
           }
         }
-      }
-      const int r0 = ((fl >> 4) << 5) + (fl & 15);  // operand row of hi; lo is 16 below
-      const int o0 = r0 * 128 + ((c ^ (r0 & 7)) << 4);
-      const int o1 = o0 + 16 * 128;  // (r0 + 16) & 7 == r0 & 7
-      *reinterpret_cast<uint4*>(img + o0) = make_uint4(p0[0], p0[1], p0[2], p0[3]);
-      *reinterpret_cast<uint4*>(img + o1) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
-      if (ext) {
-        *reinterpret_cast<uint4*>(imx + o0) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
-        *reinterpret_cast<uint4*>(imx + o1) = make_uint4(0u, 0u, 0u, 0u);
+        const int r0 = ((fl >> 4) << 5) + (fl & 15);  // operand row of hi; lo is 16 below
+        const int o0 = r0 * 128 + ((c ^ (r0 & 7)) << 4);
+        const int o1 = o0 + 16 * 128;  // (r0 + 16) & 7 == r0 & 7
+        *reinterpret_cast<uint4*>(img + o0) = make_uint4(p0[0], p0[1], p0[2], p0[3]);
+        *reinterpret_cast<uint4*>(img + o1) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
       }
     }
+    if (pair || !ext) return;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TF_FM / 8; ++i) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (lane + 32 * j < PF_GPU) al[(TF_FM / 8) * warp + i][lane + 32 * j] = split2(v[i][j], digit, frac, unfrac);
+    }
+    __syncthreads();
   }
 }
 
@@ -621,7 +646,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) fold_contract_kernel(const __gr
         }
         for (int pass = 0; pass < passes; ++pass) {
           if (!ok) continue;  // after a failed wait: run out the tile, then leave with the others
-          const float r = pass ? r0 * a.ext_scale : r0;  // the third part (in hi's rows)
+          const float r = pass ? r0 * a.ext_scale : r0;  // the second pair, below the first
           if (!mbar_wait_warp(&acc_full[b], fph, tmo, abort_flag)) {
             ok = false;
             continue;
@@ -727,6 +752,22 @@ int num_sms() {
   return sms;
 }
 
+// Whether every group lies inside one 16-element slice of a K-tile (one MMA step).
+bool in_slices(const Geom& g) { return g.G <= 16 && (g.Cg % g.G == 0 || g.R * g.S == 1); }
+
+// The share of an alpha that its first pair of parts may leave out before the unit takes the second
+// pair: so much that the output's error, with the fp32 adds of the units beside it, is no larger than
+// that of fp32 alphas on exact group sums added in fp32 (the dp4a kernel), whichever alphas the
+// activations leave active.  Measured, root mean square against 64 bits: n fp32 adds err by
+// 1.75e-8 sqrt(n) for dp4a's groups (72 1.41e-7, 288 3.0e-7, 576 4.3e-7) and 2.8e-8 sqrt(n) for the units'
+// (9 8.5e-8); a share that is uniform up to tol adds tol / sqrt(3).  G = 4 keeps 22 bits, as the
+// split per group slot that ran it before, and every G 20 (the 1e-5 of S above).
+float pair_tolerance(const Geom& g, int nunits) {
+  const double spare = g.ng - 3.0 * nunits;
+  const double tol = spare > 0.0 ? 2.7e-8 * sqrt(spare) : 0.0;
+  return g.G == 4 ? 0x1p-22f : (float)(tol < 0x1p-20 ? tol : 0x1p-20);
+}
+
 // Positions per tile: the size that makes the persistent grid's last wave cheap.  A K-tile
 // takes 2 bn clk of the tensor pipe (at least about 400 clk of issue), a tile's drain and
 // stores about 10 bn + 600 clk, which overlap the next tile's MMAs.
@@ -818,7 +859,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   const int64_t lim_us = debug_wait_limit_us();
   a.timeout_ns = lim_us < 0 ? TF_TIMEOUT_NS : (uint64_t)lim_us * 1000u;
 
-  // one temporary from the stream-ordered pool: weight images, third parts, row scales, marks,
+  // one temporary from the stream-ordered pool: weight images, second pairs, row scales, marks,
   // fp16 activations
   cudaMemPool_t pool = scratch_pool();
   if (!pool) return FGQ_ERR_CUDA;
@@ -846,6 +887,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.ng = g.ng;
   f.gshift = 31 - __builtin_clz((unsigned)g.G);
   f.dbits = g.G > 32 ? TF_DIGIT - 1 : TF_DIGIT;
+  f.fbits = in_slices(g) ? TF_FRAC : 0;
   a.lo_scale = 1.0f / (float)(1 << f.dbits);
   a.ext_scale = a.lo_scale * a.lo_scale;
   f.Mg = g.Mg;
@@ -857,7 +899,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   f.uk = a.uk;
   f.ux = a.ux;
   f.nsub = wtiles * a.nunits >= 2 * sms ? 1 : TF_UNIT;
-  f.third = g.G > 32 || (g.G > 4 && g.ng < FOLD_FEW_GROUPS) ? 1 : 0;
+  f.tol = pair_tolerance(g, a.nunits);
   f.quads = g.Cg % 4 == 0 ? 1 : 0;
   f.padded = (a.cpad != g.Cg || g.C % 16 != 0) ? 1 : 0;
   f.fast8 = f.padded && g.Cg % 8 == 0 && g.C % 8 == 0 && (g.act_type == FGQ_U8 || g.act_type == FGQ_S8) ? 1 : 0;

@@ -87,3 +87,58 @@ def test_fold_sums_inside_groups(G):
     assert fgq.fgq_last_path() == fgq.PATH_TC
     check_within(got, y, ym, f"sums inside groups G={G}")
     assert np.all(got[ym == 0] == 0)
+
+
+@pytest.mark.parametrize("ratio", [1, 2, 3, 5, 8, 45, 700, 2 ** 20])
+@pytest.mark.parametrize("G,K", [(4, 2304), (4, 256), (8, 2304), (16, 2304), (32, 2304), (32, 512), (32, 1152), (8, 9216), (64, 2336)])
+def test_fold_small_alphas_alone(G, K, ratio):
+    """One group in 256 elements has the largest alpha, `ratio` times the others', and meets channels that
+    are zero: the output's error is that of the small alphas' parts, no larger than the error of fp32
+    alphas on exact group sums (the dp4a kernel)."""
+    rng = np.random.default_rng(1000 * G + K + ratio)
+    P, M = 200, 128
+    ng = -(-K // G)
+    al = rng.uniform(1.0, 2.0, (M, ng)).astype(np.float32)
+    t = rng.integers(-1, 2, (M, ng * G)).astype(np.int8)
+    t[:, K:] = 0
+    q = rng.integers(0, 256, (P, K)).astype(np.int32)
+    for k in range(0, K, 256):
+        al[:, k // G] *= np.float32(ratio)
+        q[:, k:k + G] = 0
+    y, _ = O.gemm(q, np.float32(1.0), t, al, G)
+    q = q.reshape(P, 1, 1, K)
+    got = _conv(q, "u8", t, al, G, 1, 1, path=fgq.PATH_TC if G == 4 and K % 64 == 0 else fgq.PATH_AUTO).reshape(P, M)
+    assert fgq.fgq_last_path() == fgq.PATH_TC
+    simt = _conv(q, "u8", t, al, G, 1, 1, path=fgq.PATH_SIMT).reshape(P, M)
+    rms = np.sqrt(np.mean(y ** 2))
+    err, ref = (np.sqrt(np.mean((v.astype(np.float64) - y) ** 2)) / rms for v in (got, simt))
+    # both are sums of roundings; 1.1 and 0.05 ulp for the spread of two draws of them
+    assert err <= 1.1 * ref + 0.05 * 2.0 ** -24, (err, ref)
+
+
+@pytest.mark.parametrize("G", [4, 8, 16])
+@pytest.mark.parametrize("frac", [0, 3, 6])
+def test_fold_step_sums_are_exact(G, frac):
+    """Groups inside one MMA step: the products of a group that cancels, as large as they get, leave nothing
+    of themselves and take nothing from an alpha on the finest grid of the parts beside them."""
+    rng = np.random.default_rng(10 * G + frac)
+    P, K, M = 130, 1024, 128
+    ng = K // G
+    t = np.zeros((M, ng, G), np.int8)
+    for r in t.reshape(-1, G):
+        i = rng.permutation(G)
+        r[i[:G // 2]], r[i[G // 2:]] = 1, -1
+    al = np.full((M, ng), 2047 / 1024, np.float32)
+    al[:, ::3] = 1999 / 1024
+    for m in range(M):  # one group of one code: al is an odd multiple of 2^-frac / 1024, 10 bits long
+        g = m * ng // M
+        t[m, g] = 0
+        t[m, g, rng.integers(G)] = rng.choice([-1, 1])
+        al[m, g] = (rng.integers(2 ** 9, 2 ** 10) | 1) * 2.0 ** -frac / 1024
+    t = t.reshape(M, K)
+    q = np.full((P, K), 255, np.int32)
+    q[1::2] = rng.integers(1, 256, (P // 2, 1))
+    y, _ = O.gemm(q, np.float32(1.0), t, al, G)
+    got = _conv(q.reshape(P, 1, 1, K), "u8", t, al, G, 1, 1).reshape(P, M)
+    assert fgq.fgq_last_path() == fgq.PATH_TC
+    assert np.array_equal(got, y.astype(np.float32))

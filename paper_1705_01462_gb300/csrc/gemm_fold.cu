@@ -321,14 +321,23 @@ __global__ void __launch_bounds__(256, 4) prep_fold_kernel(const __grid_constant
 #pragma unroll
   for (int i = 0; i < TF_FM / 8; ++i) {
     const int fl = (TF_FM / 8) * warp + i;
-    float mx = 0.0f;
+    uint32_t mx = 0;  // the largest magnitude's bits: above infinity's if one is a NaN
 #pragma unroll
-    for (int j = 0; j < 3; ++j) mx = fmaxf(mx, fabsf(v[i][j]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int j = 0; j < 3; ++j) mx = max(mx, __float_as_uint(v[i][j]) & 0x7fffffffu);
+    mx = __reduce_max_sync(FULL_MASK, mx);
     // 2^e puts the largest alpha into [digit / 4, digit / 2); e is kept where 2^e and 2^-e are normal
-    int e = mx > 0.0f ? f.dbits - 2 - ilogbf(mx) : 0;
-    e = e < -120 ? -120 : (e > 120 ? 120 : e);
+    int e = 0;
+    if (mx < 0x7f800000u) {
+      if (mx != 0) e = f.dbits - 2 - ilogbf(__uint_as_float(mx));
+      e = e < -120 ? -120 : (e > 120 ? 120 : e);
+    } else {
+      // An infinite alpha: a number that both pairs hold a share of, at a row scale of infinity; the others
+      // zero.  The unit gives infinity where its codes' sum is not zero, else NaN, as infinity times
+      // the group sum does.  A NaN: a row scale of NaN.
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        v[i][j] = (__float_as_uint(v[i][j]) & 0x7fffffffu) == 0x7f800000u ? copysignf(0x1.000002p-1f, v[i][j]) : 0.0f;
+    }
     const float mul = pow2f(e);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -338,7 +347,8 @@ __global__ void __launch_bounds__(256, 4) prep_fold_kernel(const __grid_constant
       if (fabsf(v[i][j]) > tol * fabsf(x)) wide = true;
       if (lane + 32 * j < PF_GPU) al[fl][lane + 32 * j] = parts;
     }
-    if (sub == 0 && lane == 0) f.rs[((int64_t)tile * f.nunits + u) * TF_FM + fl] = pow2f(-e);
+    if (sub == 0 && lane == 0)
+      f.rs[((int64_t)tile * f.nunits + u) * TF_FM + fl] = mx < 0x7f800000u ? pow2f(-e) : __uint_as_float(mx);
   }
   const bool ext = __syncthreads_or(wide);
   if (sub == 0 && threadIdx.x == 0) f.ext[(int64_t)tile * f.nunits + u] = ext ? 1 : 0;

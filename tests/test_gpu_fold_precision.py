@@ -142,3 +142,33 @@ def test_fold_step_sums_are_exact(G, frac):
     got = _conv(q.reshape(P, 1, 1, K), "u8", t, al, G, 1, 1).reshape(P, M)
     assert fgq.fgq_last_path() == fgq.PATH_TC
     assert np.array_equal(got, y.astype(np.float32))
+
+
+@pytest.mark.parametrize("G,K", [(4, 512), (8, 2304), (16, 512), (32, 2304), (64, 2336)])
+def test_fold_nonfinite_alphas(G, K):
+    """A caller's infinite and NaN alphas, on codes and on groups without any: the outputs that they reach
+    are the dp4a kernel's (alpha s in fp32: infinite, or NaN where s is 0), the other filters' are as
+    ever."""
+    rng = np.random.default_rng(G)
+    P, M = 96, 128
+    ng = -(-K // G)
+    al = rng.uniform(0.001, 2.0, (M, ng)).astype(np.float32)
+    t = rng.integers(-1, 2, (M, ng, G)).astype(np.int8)
+    t[:, -1] = 0  # (ragged where K % G)
+    q = rng.integers(0, 256, (P, K)).astype(np.int32)
+    q[::3, :256] = 0
+    al[0, 0], al[1, 1], al[2, ng // 2] = np.inf, -np.inf, np.nan
+    al[64, 0] = al[65, 0] = np.inf
+    al[66, 1] = np.nan
+    t[64, 0] = t[66, 1] = 0  # no codes
+    t = t.reshape(M, -1)
+    clean = np.ones(M, bool)
+    clean[[0, 1, 2, 64, 65, 66]] = False
+    y, ym = O.gemm(q, np.float32(1.0), t[clean], al[clean], G)
+    q = q.reshape(P, 1, 1, K)
+    got = _conv(q, "u8", t, al, G, 1, 1).reshape(P, M)
+    assert fgq.fgq_last_path() == fgq.PATH_TC
+    simt = _conv(q, "u8", t, al, G, 1, 1, path=fgq.PATH_SIMT).reshape(P, M)
+    assert np.isnan(simt[:, [2, 64, 66]]).all() and np.isinf(simt).any()
+    assert np.array_equal(got[:, ~clean], simt[:, ~clean], equal_nan=True)
+    check_within(got[:, clean], y, ym, f"non-finite alphas beside, G={G}")

@@ -257,7 +257,8 @@ fgq_status fgq_quantize_weights_w8(const float* w, int M, int Kred, int8_t* wq, 
  * spread alphas need: 8 * M' * Kp' bytes, M' and Kp' padded to multiples of 64; the group sums
  * of G = 4 take 8 * M' * Kp bytes for a block-diagonal form instead).
  * The pool keeps freed blocks, so only a call that needs more than the pool holds reaches
- * the device allocator.  The dp4a and few-row paths allocate nothing.
+ * the device allocator.  The dp4a and few-row paths allocate nothing; where the temporary for folded
+ * weights cannot be had, the automatic choice runs on dp4a instead.
  * Errors: FGQ_ERR_ARG (null pointers, bad sizes, Kred odd for 4-bit types),
  * FGQ_ERR_ALIGN (any pointer not 16-byte aligned), FGQ_ERR_CUDA.
  */

@@ -67,6 +67,12 @@ int fgq_last_path(void);
 int64_t fgq_debug_set_wait_limit_us(int64_t us);
 
 /*
+ * Makes this thread's requests for per-call temporaries of more than `bytes` bytes fail as they do on
+ * a device without memory (bytes < 0, the default: none); returns the previous setting.
+ */
+int64_t fgq_debug_set_scratch_limit(int64_t bytes);
+
+/*
  * Lets FGQ_PATH_DENSE run calls with fp32 alphas on this thread through the split-fp16
  * ablation (allow != 0), outside the fgq_gemm tolerance; 0 restores FGQ_ERR_UNSUPPORTED.
  * Returns the previous setting.

@@ -23,6 +23,7 @@ std::atomic<uint64_t> g_launches{0};
 thread_local int t_path = FGQ_PATH_AUTO;
 thread_local int t_last_path = FGQ_PATH_AUTO;
 thread_local int64_t t_wait_limit_us = -1;
+thread_local int64_t t_scratch_limit = -1;
 thread_local int t_split_fold = 0;
 thread_local int t_last_cuda_error = 0;  // cudaError_t of the last failed launch on this thread
 thread_local int t_cta_pairs = 0;        // remembered only: every contraction kernel runs on single CTAs
@@ -145,10 +146,8 @@ fgq_status contract(const void* act, const Geom& g, const uint32_t* codes, const
                        g.rq_signed, s);
   float* a32 = nullptr;  // fixed-point alphas on the fp32-alpha kernels: alpha' = a 2^E, exact
   if (qa) {
-    cudaMemPool_t pool = scratch_pool();
-    if (!pool || cudaMallocFromPoolAsync(reinterpret_cast<void**>(&a32), sizeof(float) * (size_t)g.M * g.ng, pool, s) !=
-                     cudaSuccess)
-      return FGQ_ERR_CUDA;
+    a32 = static_cast<float*>(scratch_alloc(sizeof(float) * (size_t)g.M * g.ng, s));
+    if (!a32) return FGQ_ERR_CUDA;
     fgq_status st = launch_dequantize_alpha(qa->aq, qa->bits, g.M, g.ng, qa->ascale, a32, s);
     if (st != FGQ_OK) {
       cudaFreeAsync(a32, s);
@@ -163,13 +162,21 @@ fgq_status contract(const void* act, const Geom& g, const uint32_t* codes, const
                          : launch_fold_contract(act, g, codes, alpha, act_scale, out, err, s);
   else
     st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
+  if (st == FGQ_NO_SCRATCH) {  // the dp4a kernel needs no temporary
+    if (t_path == FGQ_PATH_AUTO) {
+      t_last_path = FGQ_PATH_SIMT;
+      st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
+    } else {
+      st = FGQ_ERR_CUDA;
+    }
+  }
   if (a32 && cudaFreeAsync(a32, s) != cudaSuccess && st == FGQ_OK) st = FGQ_ERR_CUDA;
   return st;
 }
 
 }  // namespace
 
-cudaMemPool_t scratch_pool() {
+static cudaMemPool_t scratch_pool() {
   static std::mutex mu;
   static cudaMemPool_t pools[kMaxDevices] = {};
   int dev = 0;
@@ -188,6 +195,15 @@ cudaMemPool_t scratch_pool() {
     pools[dev] = p;
   }
   return pools[dev];
+}
+
+void* scratch_alloc(size_t bytes, cudaStream_t s) {
+  if (t_scratch_limit >= 0 && bytes > (uint64_t)t_scratch_limit) return nullptr;
+  cudaMemPool_t pool = scratch_pool();
+  void* p = nullptr;
+  if (pool && cudaMallocFromPoolAsync(&p, bytes, pool, s) == cudaSuccess) return p;
+  cudaGetLastError();  // or the next launch would report it
+  return nullptr;
 }
 
 unsigned int* device_error_word() {
@@ -701,6 +717,12 @@ int fgq_set_path(int path) {
 int64_t fgq_debug_set_wait_limit_us(int64_t us) {
   const int64_t prev = t_wait_limit_us;
   t_wait_limit_us = us < 0 ? -1 : us;
+  return prev;
+}
+
+int64_t fgq_debug_set_scratch_limit(int64_t bytes) {
+  const int64_t prev = t_scratch_limit;
+  t_scratch_limit = bytes < 0 ? -1 : bytes;
   return prev;
 }
 

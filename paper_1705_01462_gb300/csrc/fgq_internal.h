@@ -131,9 +131,12 @@ fgq_status launch_add_codes(const uint8_t* a, int a_signed, const float* a_scale
                             const float* b_scale, int64_t n, float* out, uint8_t* out_q, const float* out_scale,
                             int o_signed, cudaStream_t s);
 
-// Stream-ordered memory pool of the current device for per-call temporaries (it keeps
-// freed blocks: no release threshold).  nullptr if it cannot be created.
-cudaMemPool_t scratch_pool();
+// A per-call temporary from the stream-ordered memory pool of the current device (which keeps freed
+// blocks: no release threshold); nullptr if there is none to be had, with no error left behind for
+// the next launch to report.  Returned with cudaFreeAsync on the same stream.
+void* scratch_alloc(size_t bytes, cudaStream_t s);
+// What launch_fold_contract returns in that case, before it has launched anything (never returned to a caller).
+constexpr fgq_status FGQ_NO_SCRATCH = (fgq_status)-1;
 
 // Fixed-point alphas (8- or 4-bit codes, one scale 2^E per filter row).
 fgq_status launch_quantize_alpha(const float* alpha, int M, int ng, int bits, uint8_t* aq, float* ascale,

@@ -857,14 +857,15 @@ fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t*
   if (aq ? (abits != 8 && abits != 4) || !ascale : !alpha) return FGQ_ERR_ARG;
   const int NA = aq ? 1 : 2;
   // folded weights fp16 [NA][M][Kp] and row scales [M], in one temporary from the pool
-  cudaMemPool_t pool = scratch_pool();
-  if (!pool) return FGQ_ERR_CUDA;
   const size_t part_bytes = (size_t)g.M * g.Kp * 2;
-  const bool rows = NA == 1 && tc_rows_supports(g) && !reads_once(g);  // the dense form of the G >= 64 kernel
+  bool rows = NA == 1 && tc_rows_supports(g) && !reads_once(g);  // the dense form of the G >= 64 kernel
   const size_t rs_off = NA * part_bytes, x_off = (rs_off + (size_t)g.M * 4 + 255) / 256 * 256;
-  void* tmp = nullptr;
-  if (cudaMallocFromPoolAsync(&tmp, x_off + (rows ? tc_rows_act_bytes(g) : 0), pool, s) != cudaSuccess)
-    return FGQ_ERR_CUDA;
+  void* tmp = rows ? scratch_alloc(x_off + tc_rows_act_bytes(g), s) : nullptr;
+  if (!tmp) {  // no copy of the activations, or no room for it
+    rows = false;
+    tmp = scratch_alloc(x_off, s);
+  }
+  if (!tmp) return FGQ_ERR_CUDA;
   __half* a0 = static_cast<__half*>(tmp);
   __half* a1 = NA == 2 ? a0 + (size_t)g.M * g.Kp : nullptr;
   float* rs = reinterpret_cast<float*>(static_cast<uint8_t*>(tmp) + rs_off);
@@ -901,12 +902,9 @@ fgq_status launch_dense_w8(const void* act, const Geom& g, const int8_t* wq, con
   if (!dense_w8_supports(g)) return FGQ_ERR_UNSUPPORTED;
   if (few_supports(g)) return launch_few(act, g, wq, wscale, act_scale, out, err, s);
   const int Kc = (g.Kred + TD_KT - 1) / TD_KT * TD_KT;
-  cudaMemPool_t pool = scratch_pool();
-  if (!pool) return FGQ_ERR_CUDA;
   const size_t col_bytes = (size_t)g.P * Kc, a_bytes = (size_t)g.M * Kc * 2;
-  void* tmp = nullptr;
-  if (cudaMallocFromPoolAsync(&tmp, col_bytes + a_bytes + (size_t)g.M * 4, pool, s) != cudaSuccess)
-    return FGQ_ERR_CUDA;
+  void* tmp = scratch_alloc(col_bytes + a_bytes + (size_t)g.M * 4, s);
+  if (!tmp) return FGQ_ERR_CUDA;
   uint8_t* col = static_cast<uint8_t*>(tmp);
   __half* a0 = reinterpret_cast<__half*>(col + col_bytes);
   float* rs = reinterpret_cast<float*>(col + col_bytes + a_bytes);

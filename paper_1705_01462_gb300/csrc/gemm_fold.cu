@@ -871,8 +871,6 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
 
   // one temporary from the stream-ordered pool: weight images, second pairs, row scales, marks,
   // fp16 activations
-  cudaMemPool_t pool = scratch_pool();
-  if (!pool) return FGQ_ERR_CUDA;
   const bool pointwise = tc::act_pointwise(g);
   const int64_t npix = pointwise && g.stride > 1 ? g.P : (int64_t)g.B * g.H * g.W;
   const int64_t ca = (int64_t)g.groups * a.cpad;
@@ -880,9 +878,8 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   const size_t rs_bytes = ((size_t)wtiles * a.nunits * TF_FM * 4 + 255) / 256 * 256;
   const size_t ext_bytes = ((size_t)wtiles * a.nunits + 255) / 256 * 256;
   const size_t x_bytes = (size_t)npix * ca * 2;
-  void* tmp = nullptr;
-  if (cudaMallocFromPoolAsync(&tmp, 2 * a_bytes + rs_bytes + ext_bytes + x_bytes, pool, s) != cudaSuccess)
-    return FGQ_ERR_CUDA;
+  void* tmp = scratch_alloc(2 * a_bytes + rs_bytes + ext_bytes + x_bytes, s);
+  if (!tmp) return FGQ_NO_SCRATCH;
   uint8_t* base = static_cast<uint8_t*>(tmp);
   PrepFold f;
   memset(&f, 0, sizeof f);

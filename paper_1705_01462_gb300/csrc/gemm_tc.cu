@@ -690,15 +690,11 @@ fgq_status launch_tc_contract(const void* act, const Geom& g, const uint32_t* co
   // one temporary from the stream-ordered pool: the codes expanded [M][Kp] (Kp = 16 wrow), the
   // activations expanded NHWC (a strided 1x1 convolution: only the pixels it reads, [P][C]) and the
   // transposed alphas
-  cudaMemPool_t pool = scratch_pool();
-  if (!pool) return FGQ_ERR_CUDA;
   const int64_t nwords = (int64_t)g.M * g.wrow;
   const int64_t nact = tc::act16_elems(g);
   const size_t a_bytes = ((size_t)nwords * 16 * es + 255) / 256 * 256, x_bytes = ((size_t)nact * es + 255) / 256 * 256;
-  void* a16 = nullptr;
-  if (cudaMallocFromPoolAsync(&a16, a_bytes + x_bytes + (alpha ? sizeof(float) * (size_t)g.M * g.ng : 0), pool, s) !=
-      cudaSuccess)
-    return FGQ_ERR_CUDA;
+  void* a16 = scratch_alloc(a_bytes + x_bytes + (alpha ? sizeof(float) * (size_t)g.M * g.ng : 0), s);
+  if (!a16) return FGQ_ERR_CUDA;
   void* x16 = static_cast<uint8_t*>(a16) + a_bytes;
   float* alpha_t = reinterpret_cast<float*>(static_cast<uint8_t*>(x16) + x_bytes);
   a.alpha_t = alpha_t;

@@ -370,13 +370,11 @@ fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes
 
   // one temporary from the stream-ordered pool: the block-diagonal ternary operand A' and the
   // activations in fp16
-  cudaMemPool_t pool = scratch_pool();
-  if (!pool) return FGQ_ERR_CUDA;
   const int64_t arows = (int64_t)g.groups * a.mtiles * T4_ROWS;
   const size_t diag_bytes = (size_t)arows * g.Kp * 2;
   const size_t x16_bytes = (size_t)tc::act16_elems(g) * 2;
-  void* tmp = nullptr;
-  if (cudaMallocFromPoolAsync(&tmp, diag_bytes + x16_bytes, pool, s) != cudaSuccess) return FGQ_ERR_CUDA;
+  void* tmp = scratch_alloc(diag_bytes + x16_bytes, s);
+  if (!tmp) return FGQ_ERR_CUDA;
   uint8_t* diag = static_cast<uint8_t*>(tmp);
   uint8_t* x16 = diag + diag_bytes;
   const int ksplit = (g.Kp / 8 + PREP4_CHUNKS - 1) / PREP4_CHUNKS;

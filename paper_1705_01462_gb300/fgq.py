@@ -63,6 +63,7 @@ SIGNATURES = [
     ("fgq_launch_count", _u64, []),
     ("fgq_selftest_wait_timeout", _i, [_u32, _vp]),
     ("fgq_debug_set_wait_limit_us", _i64, [_i64]),
+    ("fgq_debug_set_scratch_limit", _i64, [_i64]),
     ("fgq_debug_allow_split_fold", _i, [_i]),
     ("fgq_debug_selftest_warp_wait", _i, [_u32, _vp]),
     ("fgq_debug_last_cuda_error", _i, [_vp, _sz]),
@@ -515,6 +516,11 @@ def fgq_set_path(path: int) -> int:
 def fgq_debug_set_wait_limit_us(us: int) -> int:
     """Wait limit of this thread's tensor-core kernel launches (test control; -1 restores)."""
     return int(lib().fgq_debug_set_wait_limit_us(us))
+
+
+def fgq_debug_set_scratch_limit(nbytes: int) -> int:
+    """Per-call temporaries above `nbytes` fail on this thread (negative: none); the previous limit."""
+    return int(lib().fgq_debug_set_scratch_limit(nbytes))
 
 
 def fgq_debug_allow_split_fold(allow: bool) -> int:

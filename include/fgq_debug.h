@@ -73,6 +73,13 @@ int64_t fgq_debug_set_wait_limit_us(int64_t us);
 int64_t fgq_debug_set_scratch_limit(int64_t bytes);
 
 /*
+ * Makes this thread's cooperative launches of more than `blocks` blocks (fgq_quantize_act_batch) fail as
+ * they do in a context that can keep no more resident (blocks < 0, the default: none); returns the
+ * previous setting.
+ */
+int64_t fgq_debug_set_resident_blocks(int64_t blocks);
+
+/*
  * Lets FGQ_PATH_DENSE run calls with fp32 alphas on this thread through the split-fp16
  * ablation (allow != 0), outside the fgq_gemm tolerance; 0 restores FGQ_ERR_UNSUPPORTED.
  * Returns the previous setting.

@@ -24,6 +24,7 @@ thread_local int t_path = FGQ_PATH_AUTO;
 thread_local int t_last_path = FGQ_PATH_AUTO;
 thread_local int64_t t_wait_limit_us = -1;
 thread_local int64_t t_scratch_limit = -1;
+thread_local int64_t t_resident_blocks = -1;
 thread_local int t_split_fold = 0;
 thread_local int t_last_cuda_error = 0;  // cudaError_t of the last failed launch on this thread
 thread_local int t_cta_pairs = 0;        // remembered only: every contraction kernel runs on single CTAs
@@ -236,6 +237,8 @@ fgq_status after_launch(cudaError_t launch_result) {
 int64_t debug_wait_limit_us() { return t_wait_limit_us; }
 
 int debug_max_ksplit() { return t_max_ksplit; }
+
+int64_t debug_resident_blocks() { return t_resident_blocks; }
 
 void note_ksplit(int k) { t_last_ksplit = k; }
 
@@ -723,6 +726,12 @@ int64_t fgq_debug_set_wait_limit_us(int64_t us) {
 int64_t fgq_debug_set_scratch_limit(int64_t bytes) {
   const int64_t prev = t_scratch_limit;
   t_scratch_limit = bytes < 0 ? -1 : bytes;
+  return prev;
+}
+
+int64_t fgq_debug_set_resident_blocks(int64_t blocks) {
+  const int64_t prev = t_resident_blocks;
+  t_resident_blocks = blocks < 0 ? -1 : blocks;
   return prev;
 }
 

@@ -38,6 +38,8 @@ fgq_status after_launch(cudaError_t launch_result);  // the result of a cudaLaun
 // kernels' mbarrier waits (fgq_debug_set_wait_limit_us), or -1 for the kernels' own limits.
 int64_t debug_wait_limit_us();
 int debug_max_ksplit();    // 1 .. 8
+// Blocks that a test pretends a cooperative launch can keep resident, or -1.
+int64_t debug_resident_blocks();
 void note_ksplit(int k);   // group ranges of the G >= 64 tensor-core call just launched
 
 // Kernel launchers (each returns FGQ_OK or FGQ_ERR_CUDA / FGQ_ERR_UNSUPPORTED).

@@ -609,9 +609,7 @@ fgq_status launch_qab(int n, const float* const* x, const size_t* nelem, const i
   add(prev, nt, 2);
   if (total > INT32_MAX / 2) return FGQ_ERR_UNSUPPORTED;
   p.items = (int)total;
-  const int64_t cap = (int64_t)num_sms() * kBatchBlocks;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(total < cap ? total : cap));
   cfg.blockDim = dim3(kBatchThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -619,7 +617,16 @@ fgq_status launch_qab(int n, const float* const* x, const size_t* nelem, const i
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return after_launch(cudaLaunchKernelEx(&cfg, qab_kernel<MAXT>, p, err));
+  // A context that holds a part of the SMs (a partition of the device) cannot keep the whole grid
+  // resident: fewer blocks, down to one, do the same items.
+  const int64_t cap = (int64_t)num_sms() * kBatchBlocks, resident = debug_resident_blocks();
+  for (int64_t grid = total < cap ? total : cap;; grid = (grid + 1) / 2) {
+    cfg.gridDim = dim3((unsigned)grid);
+    const cudaError_t e = resident >= 0 && grid > resident ? cudaErrorCooperativeLaunchTooLarge
+                                                           : cudaLaunchKernelEx(&cfg, qab_kernel<MAXT>, p, err);
+    if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) return after_launch(e);
+    cudaGetLastError();
+  }
 }
 
 }  // namespace

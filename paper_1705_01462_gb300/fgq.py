@@ -64,6 +64,7 @@ SIGNATURES = [
     ("fgq_selftest_wait_timeout", _i, [_u32, _vp]),
     ("fgq_debug_set_wait_limit_us", _i64, [_i64]),
     ("fgq_debug_set_scratch_limit", _i64, [_i64]),
+    ("fgq_debug_set_resident_blocks", _i64, [_i64]),
     ("fgq_debug_allow_split_fold", _i, [_i]),
     ("fgq_debug_selftest_warp_wait", _i, [_u32, _vp]),
     ("fgq_debug_last_cuda_error", _i, [_vp, _sz]),
@@ -521,6 +522,11 @@ def fgq_debug_set_wait_limit_us(us: int) -> int:
 def fgq_debug_set_scratch_limit(nbytes: int) -> int:
     """Per-call temporaries above `nbytes` fail on this thread (negative: none); the previous limit."""
     return int(lib().fgq_debug_set_scratch_limit(nbytes))
+
+
+def fgq_debug_set_resident_blocks(blocks: int) -> int:
+    """Cooperative launches of more blocks fail on this thread (negative: none); the previous limit."""
+    return int(lib().fgq_debug_set_resident_blocks(blocks))
 
 
 def fgq_debug_allow_split_fold(allow: bool) -> int:

@@ -58,8 +58,8 @@ int fgq_last_path(void);
 
 /*
  * Shortens every mbarrier wait of the tensor-core contraction kernels launched by this
- * thread to about `us` microseconds (us < 0 restores the kernels' own limit of about one
- * second per wait), so that a test can make a wait run out on purpose: the kernel then
+ * thread, and the wait for a tensor's maximum in fgq_quantize_act_batch, to about `us`
+ * microseconds (us < 0 restores the kernels' own limits of one and two seconds per wait), so that a test can make a wait run out on purpose: the kernel then
  * records FGQ_ERR_TIMEOUT, each role leaves its loop, and the kernel waits -- with its
  * normal limits, which this setting never shortens -- for the copies and MMAs it issued,
  * frees its tensor memory and returns.  Returns the previous setting.

@@ -385,6 +385,7 @@ struct QBatch {
   QSegment seg[2 * MAXT];
   int nseg;
   int items;
+  uint64_t timeout_ns;
 };
 
 __device__ __forceinline__ uint32_t exponent_code(uint32_t mbits, int qmax) {
@@ -546,7 +547,7 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchBlocks) qab_kernel(const 
             uint64_t now;
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(now));
             if (t0 == 0) t0 = now;
-            if (now - t0 > kBatchTimeoutNs) {
+            if (now - t0 > p.timeout_ns) {
               record_error(err, FGQ_ERR_TIMEOUT);
               late = true;
               break;
@@ -609,6 +610,8 @@ fgq_status launch_qab(int n, const float* const* x, const size_t* nelem, const i
   add(prev, nt, 2);
   if (total > INT32_MAX / 2) return FGQ_ERR_UNSUPPORTED;
   p.items = (int)total;
+  const int64_t lim_us = debug_wait_limit_us();
+  p.timeout_ns = lim_us < 0 ? kBatchTimeoutNs : (uint64_t)lim_us * 1000u;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kBatchThreads);
   cfg.stream = s;

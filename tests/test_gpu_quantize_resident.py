@@ -1,5 +1,6 @@
 """The batched quantizer's cooperative launch where the context keeps fewer blocks resident than the device
-would (a test control refuses the larger launches as the runtime does)."""
+would (a test control refuses the larger launches as the runtime does), and its wait for a tensor's
+maximum, run out on purpose."""
 import numpy as np
 import pytest
 import torch
@@ -15,6 +16,7 @@ pytestmark = pytest.mark.gpu
 def _restore():
     yield
     fgq.fgq_debug_set_resident_blocks(-1)
+    fgq.fgq_debug_set_wait_limit_us(-1)
     assert fgq.fgq_stream_status() == fgq.FGQ_OK
 
 
@@ -41,3 +43,20 @@ def test_no_resident_block_is_an_error():
     q, sc = fgq.fgq_quantize_act_batch([x], ["u8"])[0]
     assert (q == 128).all() and float(sc.item()) == 2.0 ** -7
 
+
+def test_wait_for_the_maximum_expires():
+    """One tensor of more items than blocks: some block reaches its codes while another still reduces."""
+    x = torch.randn(1 << 25, device=dev(), generator=torch.Generator(device="cuda").manual_seed(5))
+    q0, s0 = fgq.fgq_quantize_act(x, "s8")
+    fgq.fgq_debug_set_wait_limit_us(0)
+    seen = []
+    for _ in range(12):
+        fgq.fgq_quantize_act_batch([x], ["s8"])
+        seen.append(fgq.fgq_stream_status())
+        if seen[-1] == fgq.FGQ_ERR_TIMEOUT:
+            break
+    assert seen[-1] == fgq.FGQ_ERR_TIMEOUT, seen
+    fgq.fgq_debug_set_wait_limit_us(-1)
+    q, s = fgq.fgq_quantize_act_batch([x], ["s8"])[0]
+    assert fgq.fgq_stream_status() == fgq.FGQ_OK
+    assert torch.equal(q, q0) and torch.equal(s, s0)

@@ -76,16 +76,22 @@ bool gemv_any(const Geom& g) { return !g.is_conv && gemv_supports((int)g.P, g.Kr
 // Layers that the folded kernel takes: G < 64, or G = 64 where the per-group kernel does not fit and
 // there are enough groups for its error to be the smaller one
 // (channels that are no multiple of 64: 5x5 with 2 x 48 channels on 27 x 27, batch 256, G = 64, dp4a
-// 1742 us a call, folded 205).  Left to the dp4a kernel: fewer filters or
+// 1742 us a call, folded 366).  Left to the dp4a kernel: fewer filters or
 // channels per conv group than fill a 64 x 64 weight image by a fair part, and layers so small
-// that dp4a, which needs no operand preparation, is done first -- its time is about 0.05 us per
-// reduction element and wave of 64 x 128 output blocks (two blocks per SM), against two launches:
-// one wave of Kred = 256 17 us a call against 23 us, of Kred = 432 33 us against 25 us, of
-// Kred = 1024 54 us against 22 us (calls back to back, host work included).
+// that dp4a, which needs no operand preparation, is done first: up to simt_wave_kred reduction
+// elements per wave of 64 x 128 output blocks (two blocks per SM).
 constexpr int FOLD_MIN_FILTERS = 64;
 constexpr int FOLD_MIN_CHANNELS = 16;
-constexpr int64_t SIMT_WAVE_KRED = 256;
 constexpr int TC_MIN_G = 64;  // from here on a group fills an MMA K-tile
+
+// One wave, us a call (back to back, host work included), the folded kernel 16 to 17.5: dp4a at G = 4, Kred =
+// 288 18.9; where it stages 8-bit codes by 16-byte loads G = 8, 288 14.9, 320 16.7, 384 18.8; G = 16, 320 14.5,
+// 384 16.7, 448 18.7; G = 32, 384 14.8, 448 16.8, 512 18.9; elsewhere G = 8, 324 27, G = 32, 324 25; 4-bit codes
+// 23 to 30 at 288.
+int64_t simt_wave_kred(const Geom& g) {
+  if (is4(g.act_type) || g.Cg % 32 != 0 || g.C % 16 != 0) return 256;
+  return g.G <= 4 ? 256 : (g.G == 8 ? 320 : (g.G == 16 ? 384 : 448));
+}
 
 bool fold_any(const Geom& g) {
   if (g.Mg < FOLD_MIN_FILTERS || g.Cg < FOLD_MIN_CHANNELS || !fold_supports(g)) return false;
@@ -97,7 +103,7 @@ bool fold_any(const Geom& g) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t blocks = (g.P + 127) / 128 * ((g.Mg + 63) / 64) * g.groups;
-  return (blocks + 2 * sms - 1) / (2 * sms) * g.Kred > SIMT_WAVE_KRED;
+  return (blocks + 2 * sms - 1) / (2 * sms) * g.Kred > simt_wave_kred(g);
 }
 
 int choose_path(const Geom& g, bool sums, bool qa) {

@@ -119,3 +119,22 @@ def test_fold_saturated_sums():
     got = fgq.fgq_gemm(to_dev(O.pack_act(q, O.U8)), "u8", to_dev(np.array([sc], np.float32)), P, K,
                        to_dev(O.pack_codes(t).view(np.int32)), to_dev(al), M, G).cpu().numpy()
     check_within(got, y, ym, "saturated sums")
+
+
+@pytest.mark.parametrize("G,act,C,R,path", [
+    (4, "u8", 256, 1, fgq.PATH_SIMT), (4, "u8", 288, 1, fgq.PATH_TC), (8, "u8", 320, 1, fgq.PATH_SIMT),
+    (8, "s8", 352, 1, fgq.PATH_TC), (16, "s8", 384, 1, fgq.PATH_SIMT), (16, "u8", 416, 1, fgq.PATH_TC),
+    (32, "u8", 448, 1, fgq.PATH_SIMT), (32, "u8", 480, 1, fgq.PATH_TC), (32, "u8", 32, 3, fgq.PATH_SIMT),
+    (32, "u8", 36, 3, fgq.PATH_TC), (32, "u4", 288, 1, fgq.PATH_TC)])
+def test_small_layers_choice(G, act, C, R, path):
+    """Both sides of the line up to which one wave of dp4a blocks is done before the folded kernel."""
+    rng = np.random.default_rng(C)
+    B, H, W, M = 1, 12, 14, 64
+    w = rng.standard_normal((M, R * R * C)).astype(np.float32)
+    t, al, codes = make_codes(w, G)
+    q, sc, packed = quantize_oracle(random_acts((B, H, W, C), act, rng), act)
+    y, ym = O.conv2d(q, sc, R, R, 1, R // 2, 1, t, al, G)
+    got = fgq.fgq_conv2d(to_dev(packed), act, to_dev(np.array([sc], np.float32)), B, H, W, C, R, R, 1, R // 2, 1,
+                         to_dev(codes.view(np.int32)), to_dev(al), M, G)
+    assert fgq.fgq_last_path() == path
+    check_within(got.cpu().numpy(), y, ym, f"small layer G={G} C={C}")

@@ -280,9 +280,11 @@ def fgq_quantize_act_batch(xs, act_types, stream=None):
     scs = [torch.empty(1, dtype=torch.float32, device=x.device) for x in xs]
     ws = torch.empty(max(4, int(lib().fgq_quantize_act_batch_workspace_bytes(n))), dtype=torch.uint8,
                      device=xs[0].device if n else "cuda")
-    arr = lambda ts: (ctypes.c_void_p * n)(*[_dev(t, t.dtype, "tensor") for t in ts])
-    _check(lib().fgq_quantize_act_batch(n, arr(xs), (ctypes.c_size_t * n)(*[x.numel() for x in xs]),
-                                        (ctypes.c_int * n)(*types), arr(qs), arr(scs), ws.data_ptr(), ws.numel(),
+    arr = lambda ptrs: (ctypes.c_void_p * n)(*ptrs)
+    px = arr([_dev(x, torch.float32, "x") for x in xs])
+    _check(lib().fgq_quantize_act_batch(n, px, (ctypes.c_size_t * n)(*[x.numel() for x in xs]),
+                                        (ctypes.c_int * n)(*types), arr([q.data_ptr() for q in qs]),
+                                        arr([sc.data_ptr() for sc in scs]), ws.data_ptr(), ws.numel(),
                                         _stream(stream)), "fgq_quantize_act_batch")
     return list(zip(qs, scs))
 

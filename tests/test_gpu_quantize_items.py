@@ -52,3 +52,10 @@ def test_item_edges(n):
         xs.append(x)
         ts.append(t)
     _check(xs, ts)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float64, torch.int32])
+def test_inputs_are_fp32(dtype):
+    """A tensor of another type would be read as fp32, an fp16 one past its end."""
+    with pytest.raises(TypeError):
+        fgq.fgq_quantize_act_batch([torch.ones(64, device=dev()), torch.ones(64, device=dev()).to(dtype)], ["u8", "u8"])

@@ -112,3 +112,54 @@ def test_short_wait_limits(family, G, R, limit_us):
     out = fgq.fgq_conv2d(*args).cpu().numpy()
     assert fgq.fgq_stream_status() == fgq.FGQ_OK
     check_within(out, y, ym, f"{family} after short limits")
+
+
+def _w8_call(B, H, W, C, M, R, stride, pad):
+    rng = np.random.default_rng(C)
+    w = rng.standard_normal((M, R * R * C)).astype(np.float32)
+    q, sc, packed = quantize_oracle(random_acts((B, H, W, C), "u8", rng), "u8")
+    wq, ws = O.quantize_weights_w8(w)
+    y, _ = O.conv2d_w8(q, sc, R, R, stride, pad, 1, wq, ws)
+    args = (to_dev(packed), "u8", to_dev(np.array([sc], np.float32)), B, H, W, C, R, R, stride, pad, 1, to_dev(wq),
+            to_dev(ws), M)
+    return lambda: fgq.fgq_conv2d_w8(*args).cpu().numpy(), y.astype(np.float32)
+
+
+def _sums_call(G, R):
+    rng = np.random.default_rng(G + R)
+    B, H, W, C, M = 4, 14, 14, 128, 64
+    t, _, codes = make_codes(rng.standard_normal((M, R * R * C)).astype(np.float32), G)
+    q, _, packed = quantize_oracle(random_acts((B, H, W, C), "s8", rng), "s8")
+    qd, cd = to_dev(packed), to_dev(codes.view(np.int32))
+
+    def call(path=fgq.PATH_TC):
+        fgq.fgq_set_path(path)
+        return fgq.fgq_conv2d_group_sums(qd, "s8", B, H, W, C, R, R, 1, R // 2, 1, cd, M, G).cpu().numpy()
+    return call, call(fgq.PATH_SIMT)
+
+
+@pytest.mark.parametrize("kernel", ["im2col_dense", "few_channels", "few_channels_s1", "sums_g4_3x3", "sums_g4_1x1",
+                                    "sums_g64"])
+def test_forced_wait_expiry_of_the_exact_kernels(kernel):
+    """The kernels whose outputs are exact integers (times one scale): the dense kernel that converts its
+    operands in flight, the few-channel one, and the group sums."""
+    call, want = {"im2col_dense": lambda: _w8_call(4, 30, 30, 16, 64, 3, 1, 1),
+                  "few_channels": lambda: _w8_call(8, 64, 64, 3, 64, 7, 2, 3),
+                  "few_channels_s1": lambda: _w8_call(8, 32, 32, 8, 130, 3, 1, 1),
+                  "sums_g4_3x3": lambda: _sums_call(4, 3), "sums_g4_1x1": lambda: _sums_call(4, 1),
+                  "sums_g64": lambda: _sums_call(64, 3)}[kernel]()
+    assert np.array_equal(call(), want)
+    fgq.fgq_debug_set_wait_limit_us(0)
+    seen = []
+    for _ in range(TRIES):
+        out = call()
+        seen.append(fgq.fgq_stream_status())
+        assert seen[-1] in (fgq.FGQ_OK, fgq.FGQ_ERR_TIMEOUT)
+        if seen[-1] == fgq.FGQ_ERR_TIMEOUT:
+            break
+        assert np.array_equal(out, want)
+    assert seen[-1] == fgq.FGQ_ERR_TIMEOUT, f"no wait of {kernel} ran out in {TRIES} calls"
+    fgq.fgq_debug_set_wait_limit_us(-1)
+    for _ in range(2):
+        assert np.array_equal(call(), want)
+        assert fgq.fgq_stream_status() == fgq.FGQ_OK

@@ -1,6 +1,5 @@
-"""The folded tensor-core kernel (G = 4, 8, 16, 32: alphas as integers on a common grid per 256
-reduction elements, in two fp16 parts, a third where a unit's alphas spread too far) against the
-oracle, inside the contraction tolerance: channel counts that are no multiple of the K-tile,
+"""The folded tensor-core kernel (G = 4, 8, 16, 32: alphas on a common grid per about 256 reduction
+elements, in one or two pairs of fp16 parts) against the oracle, inside the contraction tolerance: channel counts that are no multiple of the K-tile,
 groups that straddle filter taps, the edges of units and tiles, strided pixels, conv groups,
 4-bit codes, and alphas and activations chosen so that only small alphas contribute."""
 import zlib

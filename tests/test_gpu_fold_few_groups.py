@@ -1,4 +1,4 @@
-"""The folded kernel where a filter has few groups (G = 8 to 32: every unit carries a third part) and at
+"""The folded kernel where a filter has few groups (G = 8 to 32: units take both pairs of parts) and at
 G = 64 on channel counts that fill no whole K-tiles (18 groups or more; fewer stay on dp4a):
 against the oracle, and no further from it than the dp4a kernel is."""
 import zlib
@@ -30,8 +30,8 @@ CASES = [
     (2, 13, 13, 200, 130, 3, 1, 1, 1, 64, "s8", fgq.PATH_TC),   # 29 groups, M % 4 != 0
     (2, 13, 13, 144, 130, 4, 1, 2, 1, 128, "s8", fgq.PATH_SIMT),
     (2, 14, 14, 96, 128, 5, 1, 2, 2, 64, "s4", fgq.PATH_TC),    # conv groups of 48 channels, 4-bit codes
-    (1, 24, 24, 64, 64, 3, 1, 1, 1, 32, "u8", fgq.PATH_TC),     # 18 groups: two parts
-    (1, 24, 24, 60, 64, 3, 1, 1, 1, 32, "u8", fgq.PATH_TC),     # 17 groups: three
+    (1, 24, 24, 64, 64, 3, 1, 1, 1, 32, "u8", fgq.PATH_TC),     # 18 groups
+    (1, 24, 24, 60, 64, 3, 1, 1, 1, 32, "u8", fgq.PATH_TC),     # 17 groups
     (1, 20, 20, 272, 64, 1, 1, 0, 1, 16, "s8", fgq.PATH_TC),    # 17 groups, two units
     (1, 20, 20, 264, 64, 1, 2, 0, 1, 128, "u8", fgq.PATH_SIMT),  # 3 groups
 ]

@@ -404,8 +404,8 @@ def test_tc_forced_on_unsupported_shape():
                                   (3, 7, 7, 64, 96, 3, 3, 2, 1, 1, 4, "s8")],
                          ids=lambda c: "x".join(map(str, c)))
 def test_g4_both_kernel_families(case, path):
-    """G = 4 through the dp4a kernel and through the block-diagonal tensor-core kernel, the
-    latter on single CTAs (the default) and on CTA pairs."""
+    """G = 4 through the dp4a kernel and through the folded tensor-core kernel; the control that once put
+    a kernel on CTA pairs is remembered and changes nothing."""
     B, H, W, C, M, R, S, stride, pad, groups, G, act = case
     rng = np.random.default_rng(zlib.crc32(repr(case).encode()) + 2)
     Kred = R * S * (C // groups)

@@ -835,19 +835,25 @@ constexpr int64_t DENSE_W8_MAX_COL_BYTES = (int64_t)8 << 30;  // the im2col temp
 
 }  // namespace
 
-// Unpadded stride-1 1x1 layers and GEMMs of few filters and many rows: this kernel converts the 8-bit
-// rows in flight, the dense form of the G >= 64 kernel reads an fp16 copy (five bytes moved per
-// activation).  Measured, 8-bit alphas, this kernel against that form: 256 -> 64 on 56 x 56, batch 64,
-// 42 / 65 us; 64 -> 256 57 / 60; 512 -> 128 on 28 x 28 29 / 35; but 1024 -> 256 on 14 x 14 27 / 23;
-// 8192 rows of 1024 -> 1024 42 / 29; and where each activation is read at several taps always the
-// form: 3 x 3 at batch 64, 64 channels on 56 x 56 83 / 61, 256 on 14 x 14 59 / 25, 512 on 7 x 7 101 / 31.
+// Unpadded stride-1 1x1 layers and GEMMs that this kernel, which converts the 8-bit rows in flight, does
+// before the dense form of the G >= 64 kernel, which reads an fp16 copy (five bytes moved per activation, a
+// launch more).  Measured over 1x1 layers of 3136 to 200704 positions, 64 to 2048 channels, 64 to 1024
+// filters, 8-bit alphas, us a call, this kernel / that form:
+//  - tiles below the SMs: the launch more decides for short reductions: 12544 positions, 128 filters, 64
+//    channels 16.6 / 20.8, 256 18.9 / 20.3, 512 21.1 / 18.7, 1024 27.4 / 21.8, 2048 40.2 / 31.9;
+//  - from there on the copy, read back by one or two filter tiles, up to 256 filters: 50176 positions, 64
+//    channels, 64 filters 18.3 / 20.4, 256 filters 25.2 / 23.6; 512 channels 29.1 / 34.7, 37.4 / 44.2; 200704
+//    positions, 512 channels 60.5 / 112.9, 98.9 / 139.6; with 512 filters and 256, 512, 1024 channels
+//    114 / 124, 174 / 179, 308 / 299, with 1024 filters 212 / 199 and 332 / 275.
+// Where each activation is read at several taps always the form: 3 x 3 at batch 64, 64 channels on 56 x 56
+// 83 / 61, 256 on 14 x 14 59 / 25, 512 on 7 x 7 101 / 31.
 static bool reads_once(const Geom& g) {
-  if (g.R != 1 || g.S != 1 || g.stride != 1 || g.pad != 0 || g.M > 512) return false;
+  if (g.R != 1 || g.S != 1 || g.stride != 1 || g.pad != 0) return false;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t tiles = (int64_t)g.groups * ((g.Mg + TD_BM - 1) / TD_BM) * ((g.P + TD_BN - 1) / TD_BN);
-  return tiles >= 2 * sms || g.P * g.C >= (int64_t)16 << 20;
+  return tiles < sms ? g.Cg <= 256 : g.Mg <= 256;
 }
 
 fgq_status launch_dense_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,

@@ -23,7 +23,10 @@ def _clean_status():
 
 @pytest.mark.parametrize("case", [(80001, 64, 64, 4, "u8"), (80001, 64, 70, 8, "s8"),   # at least two whole waves
                                   (60001, 320, 64, 4, "u8"), (60001, 256, 66, 4, "s8"),  # 18 and 15 MB of rows
-                                  (257, 128, 640, 16, "u8")], ids=lambda c: "x".join(map(str, c)))
+                                  (257, 128, 640, 16, "u8"),
+                                  # fewer tiles than SMs: 256 channels and more; whole waves: 256 filters and more
+                                  (3001, 256, 130, 4, "u8"), (3001, 320, 130, 4, "s8"), (20001, 128, 256, 8, "u8"),
+                                  (20001, 128, 260, 8, "s8")], ids=lambda c: "x".join(map(str, c)))
 def test_gemm_qa_rows_exact(case):
     P, K, M, G, act = case
     rng = np.random.default_rng(zlib.crc32(repr(case).encode()))

@@ -43,7 +43,7 @@ def test_forced_wait_expiry_then_exact(family, G, R):
     q, sc, packed = quantize_oracle(x, "u8")
     geo = (B, H, W, C, R, R, 1, pad, 1)
     qd, sd, cd = to_dev(packed), to_dev(np.array([sc], np.float32)), to_dev(codes.view(np.int32))
-    if family == "dense":  # 8-bit fixed-point alphas: the dense form of the G >= 64 kernel
+    if family == "dense":  # 8-bit fixed-point alphas: 3x3 on the dense form of the G >= 64 kernel, 1x1 in flight
         a8, asc, _ = O.quantize_alpha(al, 8)
         ad, ascd = to_dev(a8.astype(np.uint8)), to_dev(asc)
 

@@ -99,9 +99,7 @@ bool fold_any(const Geom& g) {
     const int units = (g.R * g.S * ((g.Cg + 63) / 64) + 3) / 4;  // fp32 adds of the folded kernel
     if (g.ng < FOLD_FEW_GROUPS || 2 * g.ng < 5 * units) return false;
   }
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t blocks = (g.P + 127) / 128 * ((g.Mg + 63) / 64) * g.groups;
   return (blocks + 2 * sms - 1) / (2 * sms) * g.Kred > simt_wave_kred(g);
 }
@@ -202,6 +200,13 @@ static cudaMemPool_t scratch_pool() {
     pools[dev] = p;
   }
   return pools[dev];
+}
+
+int device_sms() {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
 }
 
 void* scratch_alloc(size_t bytes, cudaStream_t s) {

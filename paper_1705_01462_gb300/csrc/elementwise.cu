@@ -141,9 +141,7 @@ fgq_status launch_maxpool_u8(const uint8_t* in, int B, int H, int W, int C, int 
 fgq_status launch_add_codes(const uint8_t* a, int a_signed, const float* a_scale, const uint8_t* b, int b_signed,
                             const float* b_scale, int64_t n, float* out, uint8_t* out_q, const float* out_scale,
                             int o_signed, cudaStream_t s) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const uintptr_t bits = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) |
                          reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(out_q);
   const int64_t n16 = (bits & 15) ? 0 : n / 16;

@@ -133,6 +133,8 @@ fgq_status launch_add_codes(const uint8_t* a, int a_signed, const float* a_scale
                             const float* b_scale, int64_t n, float* out, uint8_t* out_q, const float* out_scale,
                             int o_signed, cudaStream_t s);
 
+int device_sms();  // SMs of the current device
+
 // A per-call temporary from the stream-ordered memory pool of the current device (which keeps freed
 // blocks: no release threshold); nullptr if there is none to be had, with no error left behind for
 // the next launch to report.  Returned with cudaFreeAsync on the same stream.

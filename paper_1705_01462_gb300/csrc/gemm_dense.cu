@@ -823,9 +823,7 @@ fgq_status run_dense(const void* act, const Geom& g, int NA, const __half* a0, c
                             (uint64_t)g.M * 4, TD_BM, 64, CU_TENSOR_MAP_SWIZZLE_NONE)
                     ? 1
                     : 0;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int grid = a.ntiles < sms ? a.ntiles : sms;
   const bool sgn = g.act_type == FGQ_S8;
   return NA == 1 ? launch_dense_na<1>(a, sgn, tmap, grid, s) : launch_dense_na<2>(a, sgn, tmap, grid, s);
@@ -849,9 +847,7 @@ constexpr int64_t DENSE_W8_MAX_COL_BYTES = (int64_t)8 << 30;  // the im2col temp
 // 83 / 61, 256 on 14 x 14 59 / 25, 512 on 7 x 7 101 / 31.
 static bool reads_once(const Geom& g) {
   if (g.R != 1 || g.S != 1 || g.stride != 1 || g.pad != 0) return false;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t tiles = (int64_t)g.groups * ((g.Mg + TD_BM - 1) / TD_BM) * ((g.P + TD_BN - 1) / TD_BN);
   return tiles < sms ? g.Cg <= 256 : g.Mg <= 256;
 }

@@ -428,13 +428,6 @@ bool plan_few(const Geom& g, FewArgs& a, int sms) {
   return best < 1e30;
 }
 
-int few_sms() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 template <int CP, bool RQ, int OBUFS>
 fgq_status launch_few_kernel(const FewArgs& a, dim3 grid, int smem, cudaStream_t s) {
   if (!tc::smem_attr_once<few_kernel<CP, RQ, OBUFS>>(FW_SMEM)) return FGQ_ERR_CUDA;
@@ -453,14 +446,14 @@ fgq_status launch_few_cp(const FewArgs& a, dim3 grid, int smem, cudaStream_t s) 
 
 bool few_supports(const Geom& g) {
   FewArgs a;
-  return tc::encode_tiled() != nullptr && plan_few(g, a, few_sms());
+  return tc::encode_tiled() != nullptr && plan_few(g, a, device_sms());
 }
 
 fgq_status launch_few(const void* act, const Geom& g, const int8_t* wq, const float* wscale, const float* act_scale,
                       float* out, unsigned int* err, cudaStream_t s) {
   FewArgs a;
   memset(&a, 0, sizeof a);
-  if (!plan_few(g, a, few_sms())) return FGQ_ERR_UNSUPPORTED;
+  if (!plan_few(g, a, device_sms())) return FGQ_ERR_UNSUPPORTED;
   a.act = static_cast<const uint8_t*>(act);
   a.wq = wq;
   a.wscale = wscale;

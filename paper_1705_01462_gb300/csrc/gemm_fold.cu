@@ -755,13 +755,6 @@ fgq_status launch_fold(const FoldArgs& args, int grid, cudaStream_t s) {
   return after_launch(launch_pdl(fold_contract_kernel<TMAP, RQ>, dim3(grid), dim3(TF_THREADS), TF_SMEM, s, args));
 }
 
-int num_sms() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 // Whether every group lies inside one 16-element slice of a K-tile (one MMA step).
 bool in_slices(const Geom& g) { return g.G <= 16 && (g.Cg % g.G == 0 || g.R * g.S == 1); }
 
@@ -856,7 +849,7 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   a.nunits = (a.ktiles + a.uk - 1) / a.uk;
   a.mtiles = (g.Mg + TF_FM - 1) / TF_FM;
   const int wtiles = g.groups * a.mtiles;
-  const int sms = num_sms();
+  const int sms = device_sms();
   a.bn = choose_bn(g.P, wtiles, a.ktiles, sms);
   const int stage = TF_A + a.bn * TF_KT * 2;
   a.obufs = a.ktiles <= TF_SHORT ? 4 : 2;

@@ -632,13 +632,6 @@ void plan_tiles(TcArgs& a, const Geom& g, bool f8, int sms, bool may_split) {
 
 namespace {
 
-int device_sms() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 // Ring depth, accumulators, output boxes and wait limit once the tile size is known.
 void finish_plan(TcArgs& a, int row) {  // row: operand bytes per row of a K-tile
   const int stage = (TC_BM + a.bn) * row;

@@ -389,9 +389,7 @@ fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes
     st = FGQ_ERR_CUDA;
   if (st == FGQ_OK && !tc::act16_map(&a.act_map, x16, g, T4_BN)) st = FGQ_ERR_CUDA;
   if (st == FGQ_OK) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     const int grid = a.ntiles < sms ? a.ntiles : sms;
     st = tc::act_pointwise(g) ? launch_tc4<true>(a, grid, s) : launch_tc4<false>(a, grid, s);
   }

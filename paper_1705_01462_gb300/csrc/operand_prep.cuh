@@ -222,9 +222,7 @@ __device__ __forceinline__ void codes_e4m3(const uint32_t* codes, int64_t i, uin
 // Blocks of 256 threads for n work items: up to a full device (8 blocks of 256 threads per
 // SM), each thread looping.
 inline int blocks_for(int64_t n) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t want = (n + 255) / 256;
   return (int)(want < 8LL * sms ? (want > 0 ? want : 1) : 8LL * sms);
 }

@@ -204,16 +204,9 @@ __global__ void __launch_bounds__(kThreads) qa_quant_kernel(const float* __restr
   }
 }
 
-int num_sms() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 int max_blocks(size_t n) {
   const size_t need = (n / 16 + kThreads - 1) / kThreads;
-  const size_t cap = (size_t)num_sms() * 8;
+  const size_t cap = (size_t)device_sms() * 8;
   return (int)(need < 1 ? 1 : (need < cap ? need : cap));
 }
 
@@ -622,7 +615,7 @@ fgq_status launch_qab(int n, const float* const* x, const size_t* nelem, const i
   cfg.numAttrs = 1;
   // A context that holds a part of the SMs (a partition of the device) cannot keep the whole grid
   // resident: fewer blocks, down to one, do the same items.
-  const int64_t cap = (int64_t)num_sms() * kBatchBlocks, resident = debug_resident_blocks();
+  const int64_t cap = (int64_t)device_sms() * kBatchBlocks, resident = debug_resident_blocks();
   for (int64_t grid = total < cap ? total : cap;; grid = (grid + 1) / 2) {
     cfg.gridDim = dim3((unsigned)grid);
     const cudaError_t e = resident >= 0 && grid > resident ? cudaErrorCooperativeLaunchTooLarge

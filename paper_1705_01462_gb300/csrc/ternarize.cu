@@ -642,9 +642,7 @@ __global__ void __launch_bounds__(256) quantize_w8_kernel(const float* __restric
 }
 
 int grid_for(int64_t work_items, int threads) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int64_t need = (work_items + threads - 1) / threads;
   const int64_t cap = (int64_t)sms * 16;
   return (int)(need < 1 ? 1 : (need < cap ? need : cap));

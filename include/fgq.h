@@ -248,14 +248,19 @@ fgq_status fgq_quantize_weights_w8(const float* w, int M, int Kred, int8_t* wq, 
  *   act_scale  device fp32 [1] (e.g. the scale_out of fgq_quantize_act).
  *   codes, alpha as produced by fgq_ternarize for (M, Kred, G).
  *   y          out, fp32 [P][M].
- * The fp32 result is within 1e-5 * act_scale * sum_g |alpha_g * s_g| of the exact value.
+ * The fp32 result is within 1e-5 * act_scale * sum_g |alpha_g * s_g| of the exact value (on the
+ * folded tensor-core path, which keeps 18 bits of an alpha 2^-29 times the largest one within about 256
+ * products of its filter and fewer of still smaller ones, as far as the alphas stay above that).
  * Memory: the tensor-core kernels take per-call temporaries from a library-owned
  * stream-ordered pool of the current device and return them on the same stream: the
- * activations as fp16 (2 bytes per element read; for G < 64 each conv group's channels padded
- * to a multiple of 64), and the ternary operand -- at G >= 64 the codes as fp16 (2 * M * Kp
- * bytes) and the alphas transposed (4 * M * ng bytes), for G < 64 the folded weights (two fp16 parts, and room for the parts that widely
- * spread alphas need: 8 * M' * Kp' bytes, M' and Kp' padded to multiples of 64; the group sums
- * of G = 4 take 8 * M' * Kp bytes for a block-diagonal form instead).
+ * activations as fp16 (2 bytes per element read, 1 for 4-bit types at G >= 64), and the ternary
+ * operand.  At G >= 64 with channels per conv group a multiple of 64 that is the codes in the same
+ * type (2 or 1 bytes * M * Kp) and the alphas transposed (4 * M * ng bytes).  For G = 4 to 32, and G = 64 on
+ * other channel counts, it is the folded weights (a pair of fp16 parts, and room for the second pair
+ * that some alphas need: 8 * M' * Kp' bytes, M' padded to a multiple of 64, Kp' by each tap's channels
+ * padded so, and a quarter more where groups run past a stretch of 256 elements); the
+ * activations' channels are then padded to a multiple of 64 too.  The group sums of G = 4 take
+ * 8 * M' * Kp bytes for a block-diagonal form instead.
  * The pool keeps freed blocks, so only a call that needs more than the pool holds reaches
  * the device allocator.  The dp4a and few-row paths allocate nothing; where the temporary for folded
  * weights cannot be had, the automatic choice runs on dp4a instead.

@@ -20,15 +20,17 @@ extern "C" {
 typedef enum {
   FGQ_PATH_AUTO = 0,   /* choose per shape: the few-row path for small GEMMs; with
                           fixed-point alphas the dense tensor-core path where it applies;
-                          else the tensor cores where the shape is covered (G < 64 only with
-                          at least 64 filters and 16 channels per conv group, and not the
+                          else the tensor cores where the shape is covered (G < 64, and G = 64
+                          on channels that are no multiple of 64 with 18 groups or more, only
+                          with at least 64 filters and 16 channels per conv group, and not the
                           smallest layers), else the CUDA cores */
   FGQ_PATH_SIMT = 1,   /* CUDA-core path: dp4a group sums, one FMA per group */
   FGQ_PATH_TC = 2,     /* tensor-core path (tcgen05): G in {64, 128} with K-tiles aligned to
-                          the group; smaller G with the alphas folded into integer weights on a
-                          common grid per 256 reduction elements (two fp16 parts).  Forced: G in
-                          {4, 64, 128} with Cg a multiple of 64; the automatic choice also takes
-                          it for G = 8, 16, 32 and other channel counts */
+                          the group; smaller G with the alphas folded into the weights on a
+                          common grid per about 256 reduction elements (one or two pairs of
+                          fp16 parts).  Forced: G in {4, 64, 128} with Cg a multiple of 64; the
+                          automatic choice also takes it for G = 8, 16, 32 and other channel
+                          counts */
   FGQ_PATH_GEMV = 3,   /* few-row path for GEMMs with P <= 8 (8-bit activations, Kred a
                           multiple of 16, G >= 4): one warp per filter row streams the
                           weights once; the automatic choice for such calls */

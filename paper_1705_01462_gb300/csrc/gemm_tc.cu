@@ -121,7 +121,7 @@ struct TcArgs {
   int out_tma;      // output boxes by TMA store
   int bn, nst;      // positions per tile, ring depth
   int nacc;         // TMEM accumulator buffers of bn columns
-  int obufs;        // output boxes per epilogue warp: 1 or 2
+  int obufs;        // output boxes per epilogue warp: 2 or 4
   uint64_t timeout_ns;
 };
 

@@ -102,9 +102,11 @@ def source_digest():
 
 
 def load_traffic(digest=None):
-    """Per-call DRAM bytes from the committed ncu summaries (profiles/*traffic*.txt): lines
+    """Per-call DRAM bytes from ncu summaries of single kernels (profiles/*traffic*.txt): lines
     'family  bytes_per_call  ...' after a line '# sources <digest>'.  With `digest`, a file
-    taken from other sources contributes nothing."""
+    taken from other sources contributes nothing.  No summary is needed: without one
+    `roofline.traffic` is null.  DRAM counters belong on one kernel, a few launches and a
+    small batch (--layer, --batch), never on the whole step."""
     out = {}
     pdir = os.path.join(ROOT, "profiles")
     if not os.path.isdir(pdir):

@@ -372,7 +372,8 @@ __global__ void __launch_bounds__(NT, FGQ_SIMT_MIN_BLOCKS) simt_contract_kernel(
   if (SUMS) return;
   const float sx = __ldg(act_scale);
   const int m = mlo + ty * 4;
-  const bool vec = (g.M % 4 == 0) && (m + 3 < mhi);
+  // four outputs in one store: the row pitch and the first filter (a conv group's need not be) multiples of 4
+  const bool vec = g.M % 4 == 0 && m % 4 == 0 && m + 3 < mhi;
   if (g.rq_out) {  // fused requantization: 8-bit codes instead of fp32
     const RqMul r = rq_mul(g.rq_scale, g.rq_signed);
 #pragma unroll

@@ -161,19 +161,16 @@ fgq_status contract(const void* act, const Geom& g, const uint32_t* codes, const
     alpha = a32;
   }
   fgq_status st;
+  bool no_scratch = false;
   if (path == FGQ_PATH_TC)
     st = g.G >= TC_MIN_G && tc_supports(g) ? launch_tc_contract(act, g, codes, alpha, act_scale, out, sums, err, s)
          : sums          ? launch_tc4_sums(act, g, codes, sums, err, s)
-                         : launch_fold_contract(act, g, codes, alpha, act_scale, out, err, s);
+                         : launch_fold_contract(act, g, codes, alpha, act_scale, out, err, s, no_scratch);
   else
     st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
-  if (st == FGQ_NO_SCRATCH) {  // the dp4a kernel needs no temporary
-    if (t_path == FGQ_PATH_AUTO) {
-      t_last_path = FGQ_PATH_SIMT;
-      st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
-    } else {
-      st = FGQ_ERR_CUDA;
-    }
+  if (no_scratch && t_path == FGQ_PATH_AUTO) {  // the dp4a kernel needs no temporary
+    t_last_path = FGQ_PATH_SIMT;
+    st = launch_simt_contract(act, g, codes, alpha, 0, act_scale, out, sums, s);
   }
   if (a32 && cudaFreeAsync(a32, s) != cudaSuccess && st == FGQ_OK) st = FGQ_ERR_CUDA;
   return st;

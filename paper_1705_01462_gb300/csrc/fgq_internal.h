@@ -106,8 +106,10 @@ fgq_status launch_tc4_sums(const void* act, const Geom& g, const uint32_t* codes
 // 29 9.6e-8 / 7.3e-8, 50 12.5e-8 / 9.1e-8.
 constexpr int FOLD_FEW_GROUPS = 18;
 bool fold_supports(const Geom& g);
+// no_scratch: set where the temporary could not be had (FGQ_ERR_CUDA, nothing launched).
 fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
-                                const float* act_scale, float* out, unsigned int* err, cudaStream_t s);
+                                const float* act_scale, float* out, unsigned int* err, cudaStream_t s,
+                                bool& no_scratch);
 
 // Dense tensor-core contraction with the alphas folded into fp16 weights: fixed-point alphas
 // (aq, abits 8 or 4, ascale) exactly, or fp32 alphas (aq == nullptr) split into two fp16
@@ -139,8 +141,6 @@ int device_sms();  // SMs of the current device
 // blocks: no release threshold); nullptr if there is none to be had, with no error left behind for
 // the next launch to report.  Returned with cudaFreeAsync on the same stream.
 void* scratch_alloc(size_t bytes, cudaStream_t s);
-// What launch_fold_contract returns in that case, before it has launched anything (never returned to a caller).
-constexpr fgq_status FGQ_NO_SCRATCH = (fgq_status)-1;
 
 // Fixed-point alphas (8- or 4-bit codes, one scale 2^E per filter row).
 fgq_status launch_quantize_alpha(const float* alpha, int M, int ng, int bits, uint8_t* aq, float* ascale,

@@ -835,7 +835,8 @@ bool fold_supports(const Geom& g) {
 }
 
 fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* codes, const float* alpha,
-                                const float* act_scale, float* out, unsigned int* err, cudaStream_t s) {
+                                const float* act_scale, float* out, unsigned int* err, cudaStream_t s,
+                                bool& no_scratch) {
   if (!fold_supports(g)) return FGQ_ERR_UNSUPPORTED;
   FoldArgs a;
   memset(&a, 0, sizeof a);
@@ -872,7 +873,8 @@ fgq_status launch_fold_contract(const void* act, const Geom& g, const uint32_t* 
   const size_t ext_bytes = ((size_t)wtiles * a.nunits + 255) / 256 * 256;
   const size_t x_bytes = (size_t)npix * ca * 2;
   void* tmp = scratch_alloc(2 * a_bytes + rs_bytes + ext_bytes + x_bytes, s);
-  if (!tmp) return FGQ_NO_SCRATCH;
+  no_scratch = !tmp;
+  if (!tmp) return FGQ_ERR_CUDA;
   uint8_t* base = static_cast<uint8_t*>(tmp);
   PrepFold f;
   memset(&f, 0, sizeof f);
